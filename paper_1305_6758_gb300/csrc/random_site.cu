@@ -118,8 +118,10 @@ __global__ void __launch_bounds__(128) random_site_kernel(const SweepParams P, i
   const uint32_t sys_hi = static_cast<uint32_t>(k) << 8;
   const int init = path_init_mode(P.init_mode, path, Pk);
   for (int i = 0; i < N; ++i) {
-    Real x, y, z;
-    initial_spin<Real>(static_cast<uint32_t>(i), c2, kTagInit | sys_hi, P, init, x, y, z);
+    const Philox4 r = philox4x32_10(static_cast<uint32_t>(i), 0u, c2, kTagInit | sys_hi, P.key);
+    Real x = Real(0), y = Real(0), z = Real(1);
+    if (init == MP_INIT_ANGLES) A::init_angles(r.x, r.y, x, y, z);
+    else if (init != MP_INIT_ORDERED) A::trial(r.x, r.y, x, y, z);
     S.st(el(i), x, y, z);
   }
   const Real J = static_cast<Real>(sy.J), hf = static_cast<Real>(sy.h);

@@ -26,6 +26,7 @@
 #include <cstdint>
 
 #include "common.cuh"
+#include "fixed64.cuh"
 #include "philox.cuh"
 
 namespace mpk {
@@ -232,47 +233,82 @@ __device__ __forceinline__ void group_sync(int tp, int bar) {
 }
 
 // ------------------------------------------------------- one attempt -----
-// Per-thread partial sums of the measurement of one sweep.
-template <typename Real>
-struct Partials {
-  Real eb, mx, my, mz;
+// A 96-bit integer sum.
+struct Wide {
+  uint32_t w0 = 0, w1 = 0, w2 = 0;
+  __device__ __forceinline__ void add(uint32_t a, uint32_t b, uint32_t c) {
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        : "+r"(w0), "+r"(w1), "+r"(w2)
+        : "r"(a), "r"(b), "r"(c));
+  }
+  __device__ __forceinline__ void add(int64_t v) {
+    const uint32_t hi = static_cast<uint32_t>(static_cast<uint64_t>(v) >> 32);
+    add(static_cast<uint32_t>(v), hi, static_cast<uint32_t>(static_cast<int32_t>(hi) >> 31));
+  }
+  __device__ __forceinline__ void add_lane(int o) {  // a butterfly step over the warp
+    const uint32_t a = __shfl_xor_sync(0xffffffffu, w0, o), b = __shfl_xor_sync(0xffffffffu, w1, o),
+                   c = __shfl_xor_sync(0xffffffffu, w2, o);
+    add(a, b, c);
+  }
 };
 
+// Per-thread partial sums of the measurement of one sweep: sums of S . h over
+// the colour-1 sites and of the new spins.  FP64 form: exact integers, the
+// spins in units of 2^-53 and S . h in units of 2^-57.
+template <typename Real>
+struct Partials {
+  Real eb{}, mx{}, my{}, mz{};
+};
+template <>
+struct Partials<double> {
+  Wide eb, mx, my, mz;
+};
+constexpr double kEnergyUnit = 0x1p-57, kSpinUnit = 0x1p-53;
+
 // ------------------------------------------------------------ spin views --
+// A spin component as the kernels store it: float, or (FP64 form) the 64-bit
+// integer of fixed64.cuh.  Saved states and read-out spins are doubles.
+template <typename Real>
+struct Stored;
+template <>
+struct Stored<float> {
+  using C = float;
+  using P2 = float2;
+  static __device__ __forceinline__ C from(float v) { return v; }
+  static __device__ __forceinline__ float real(C v) { return v; }
+};
+template <>
+struct Stored<double> {
+  using C = int64_t;
+  using P2 = longlong2;
+  static __device__ __forceinline__ C from(double v) { return __double2ll_rn(v * 0x1p53); }
+  static __device__ __forceinline__ double real(C v) { return static_cast<double>(v) * kSpinUnit; }
+};
+
 template <typename Real>
 struct V3 {
-  Real x, y, z;
+  typename Stored<Real>::C x, y, z;
 };
 template <typename Real>
 __device__ __forceinline__ V3<Real> add3(V3<Real> a, V3<Real> b) {
-  using A = Arith<Real>;
-  return V3<Real>{A::add(a.x, b.x), A::add(a.y, b.y), A::add(a.z, b.z)};
+  return V3<Real>{a.x + b.x, a.y + b.y, a.z + b.z};
 }
-template <typename Real>
-struct PairOf;
-template <>
-struct PairOf<float> {
-  using T = float2;
-};
-template <>
-struct PairOf<double> {
-  using T = double2;
-};
 
 // S spins of one colour (or one half-plane): their (x, y) pairs, then their z
 // components.  base must be aligned to a pair and S even.
 template <typename Real>
 struct SpinView {
-  using P2 = typename PairOf<Real>::T;
+  using C = typename Stored<Real>::C;
+  using P2 = typename Stored<Real>::P2;
   P2* xy;
-  Real* z;
+  C* z;
   __device__ __forceinline__ SpinView(Real* base, int S)
-      : xy(reinterpret_cast<P2*>(base)), z(base + 2 * S) {}
+      : xy(reinterpret_cast<P2*>(base)), z(reinterpret_cast<C*>(base) + 2 * S) {}
   __device__ __forceinline__ V3<Real> ld(int h) const {
     const P2 v = xy[h];
     return V3<Real>{v.x, v.y, z[h]};
   }
-  __device__ __forceinline__ void st(int h, Real a, Real b, Real c) const {
+  __device__ __forceinline__ void st(int h, C a, C b, C c) const {
     P2 v;
     v.x = a;
     v.y = b;
@@ -281,21 +317,74 @@ struct SpinView {
   }
 };
 
+// | |S| - 1 | of a stored spin.
+__device__ __forceinline__ float norm_error(V3<float> v) {
+  return fabs(sqrt(v.x * v.x + v.y * v.y + v.z * v.z) - 1.0f);
+}
+__device__ __forceinline__ double norm_error(V3<double> v) {
+  // |S|^2 - 1 in units of 2^-60 from the high halves of the squares; for a
+  // unit spin |S| - 1 is half of it (one FP64 square root costs 570 cycles)
+  const int64_t a = v.x << 9, b = v.y << 9, c = v.z << 9;
+  const int64_t d = __mul64hi(a, a) + __mul64hi(b, b) + __mul64hi(c, c) - (int64_t{1} << 60);
+  const double t = static_cast<double>(d < 0 ? -d : d) * 0x1p-61;
+  if (t < 0x1p-30) return t;
+  const double x = Stored<double>::real(v.x), y = Stored<double>::real(v.y), z = Stored<double>::real(v.z);
+  return fabs(sqrt(x * x + y * y + z * z) - 1.0);  // a restored state that holds no unit spin
+}
+
+// --------------------------------------------------------- sine table ----
+// The table of fix_trial in the CTA's shared memory (FP64 kernels).
+static __device__ const SineTable kSineTable = make_sine_table();
+__device__ __forceinline__ uint64_t* sine_shared() {
+  __shared__ uint64_t t[256];
+  return t;
+}
+
+// ------------------------------------------------------------ couplings --
+// What the accept test of a path needs of its system.
+template <typename Real>
+struct Couplings;
+template <>
+struct Couplings<float> {
+  float J, hf, bp;
+  __device__ explicit Couplings(const DevSystem* s)
+      : J(static_cast<float>(s->J)), hf(static_cast<float>(s->h)), bp(Arith<float>::beta_param(s->beta)) {}
+};
+template <>
+struct Couplings<double> {
+  const DevSystem* sys;
+  float cj, ch;    // log2 of the acceptance is cj d.h + ch d_z, d and h in units of 2^-28
+  float lo, hi;    // 1 -+ the bound on the relative error of the FP32 acceptance
+  __device__ explicit Couplings(const DevSystem* s) : sys(s) {
+    const double bj = s->beta * s->J, bh = s->beta * s->h;
+    cj = static_cast<float>(bj * 1.4426950408889634 * 0x1p-56);
+    ch = static_cast<float>(bh * 1.4426950408889634 * 0x1p-28);
+    // Bound: |d| <= 2, |h| <= 6; a trial component is off by at most 1.2e-6
+    // (2^-21.2 of the hardware sine and cosine, 2^-23 of their argument, 2^-22
+    // of the radius), d by 1.5e-6, h by 3.7e-7, so d.h by 1.9e-5; the exponent's
+    // own roundings are 2^-21 of at most 33 (beyond that the test is decided),
+    // ex2 and the uniform add 2^-22.  Taken a third larger.
+    const float tol = static_cast<float>(2.5e-5 * fabs(bj) + 3e-6 * fabs(bh) + 2e-5);
+    lo = 1.0f - tol;
+    hi = 1.0f + tol;
+  }
+};
+
 // The Metropolis step at site i (half index hh of the colour view `own`)
-// given its local field (hx, hy, hz), Sec. 2.2: trial spin, energy change
-// from the local field, acceptance test.
-template <typename Real, bool kMeas, bool kEnergy>
-__device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key, const SpinView<Real>& own, int hh,
-                                       Real hx, Real hy, Real hz, Real J, Real hf, Real bp,
-                                       int& accepted, Partials<Real>& part) {
-  using A = Arith<Real>;
+// given its local field f, Sec. 2.2: trial spin, energy change from the local
+// field, acceptance test.
+template <bool kMeas, bool kEnergy>
+__device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
+                                       const SpinView<float>& own, int hh, V3<float> f,
+                                       const Couplings<float>& cp, int& accepted, Partials<float>& part) {
+  using A = Arith<float>;
   const Philox4 r = philox4x32_10(i, pre, key);
-  Real tx, ty, tz;
+  float tx, ty, tz;
   A::trial(r.x, r.y, tx, ty, tz);
-  const V3<Real> a = own.ld(hh);
-  const Real ax = a.x, ay = a.y, az = a.z;
-  Real nx = ax, ny = ay, nz = az;
-  if (A::accept_move(tx - ax, ty - ay, tz - az, hx, hy, hz, J, hf, bp, r.z)) {
+  const V3<float> a = own.ld(hh);
+  const float ax = a.x, ay = a.y, az = a.z;
+  float nx = ax, ny = ay, nz = az;
+  if (A::accept_move(tx - ax, ty - ay, tz - az, f.x, f.y, f.z, cp.J, cp.hf, cp.bp, r.z)) {
     own.st(hh, tx, ty, tz);
     nx = tx;
     ny = ty;
@@ -306,7 +395,65 @@ __device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, cons
     part.mx += nx;
     part.my += ny;
     part.mz += nz;
-    if (kEnergy) part.eb += nx * hx + ny * hy + nz * hz;
+    if (kEnergy) part.eb += nx * f.x + ny * f.y + nz * f.z;
+  }
+}
+
+// The accept test in FP64, for moves whose FP32 acceptance is too close to
+// the uniform to decide: d and h in units of 2^-53.
+static __device__ __noinline__ bool accept_exact(int64_t dx, int64_t dy, int64_t dz, int64_t hx, int64_t hy, int64_t hz,
+                                          const DevSystem* sys, uint32_t r2) {
+  using A = Arith<double>;
+  using S = Stored<double>;
+  return A::accept_move(S::real(dx), S::real(dy), S::real(dz), S::real(hx), S::real(hy), S::real(hz), sys->J,
+                        sys->h, sys->beta, r2);
+}
+
+// FP64 form.  What bounds it is FP64 issue (76 cycles per warp instruction
+// and scheduler), so none is left on the common path: the local field is an
+// integer sum, the accept test u < exp(-beta dE) is decided in FP32 wherever u
+// lies outside the FP32 acceptance's error bound (all but about 1e-5 of the
+// moves; those take accept_exact), and the trial spin is evaluated to 2^-53 in
+// integers (fix_trial), by warps in which a move was accepted.  L = 16, three
+// temperatures of 1024 paths: 5.2e9 attempts/s with FP64 arithmetic, 5.5e10 so.
+template <bool kMeas, bool kEnergy>
+__device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
+                                       const SpinView<double>& own, int hh, V3<double> f,
+                                       const Couplings<double>& cp, int& accepted, Partials<double>& part) {
+  const Philox4 r = philox4x32_10(i, pre, key);
+  const V3<double> a = own.ld(hh);
+  const FixRoot q = fix_root(r.x);
+  // d and h in units of 2^-28, as floats
+  auto f28 = [](int64_t v) { return static_cast<float>(static_cast<int32_t>(v >> 25)); };
+  const float rad = q.nf * q.y * 0x1p-4f;  // sqrt(n) 2^-32 2^28
+  float sp, cph;
+  // phi - pi = (r1 + 1/2 - 2^31) 2 pi 2^-32; sine and cosine change sign
+  __sincosf(static_cast<float>(static_cast<int32_t>(r.y ^ 0x80000000u)) * 1.46291808e-9f, &sp, &cph);
+  const float dx = -rad * cph - f28(a.x), dy = -rad * sp - f28(a.y);
+  const float dz = static_cast<float>(static_cast<int32_t>(r.x ^ 0x80000000u)) * 0.125f - f28(a.z);
+  const float dot = dx * f28(f.x) + dy * f28(f.y) + dz * f28(f.z);
+  float p;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(fmaf(cp.cj, dot, cp.ch * dz)));
+  const float u = fmaf(static_cast<float>(r.z), 0x1p-32f, 0x1p-33f);
+  bool ok = u < p * cp.lo;
+  const bool open = !ok && !(u > p * cp.hi);  // undecided (NaN and infinity included)
+  V3<double> n = a;
+  if (ok || open) {
+    const Fix3 t = fix_trial(r.x, r.y, q, sine_shared());
+    if (open) ok = accept_exact(t.x - a.x, t.y - a.y, t.z - a.z, f.x, f.y, f.z, cp.sys, r.z);
+    if (ok) {
+      own.st(hh, t.x, t.y, t.z);
+      n = V3<double>{t.x, t.y, t.z};
+      ++accepted;
+    }
+  }
+  if (kMeas) {
+    part.mx.add(n.x);
+    part.my.add(n.y);
+    part.mz.add(n.z);
+    // S . h in units of 2^-57: (S 2^62) (h 2^59) 2^-64
+    if (kEnergy)
+      part.eb.add(__mul64hi(n.x << 9, f.x << 6) + __mul64hi(n.y << 9, f.y << 6) + __mul64hi(n.z << 9, f.z << 6));
   }
 }
 
@@ -315,15 +462,14 @@ __device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, cons
 template <typename Real, int NNB, bool kMeas, bool kEnergy>
 __device__ __forceinline__ void attempt(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key, const SpinView<Real>& own,
                                         const SpinView<Real>& oth, int hh, const int* nb, int nn,
-                                        Real J, Real hf, Real bp, int& accepted,
+                                        const Couplings<Real>& cp, int& accepted,
                                         Partials<Real>& part) {
-  V3<Real> f{Real(0), Real(0), Real(0)};
+  V3<Real> f{};
 #pragma unroll
   for (int j = 0; j < NNB; ++j) {
     if (j < nn) f = add3(f, oth.ld(nb[j]));
   }
-  update<Real, kMeas, kEnergy>(i, pre, key, own, hh, f.x, f.y, f.z, J, hf, bp, accepted,
-                               part);
+  update<kMeas, kEnergy>(i, pre, key, own, hh, f, cp, accepted, part);
 }
 
 // The column chunk U of a geometry (column_chunk in common.cuh).
@@ -351,7 +497,7 @@ constexpr int kColumnChunk = column_chunk(static_cast<int>(sizeof(Real)), 2 * Ge
 template <typename Real, class Geom, bool kMeas, bool kEnergy>
 __device__ __forceinline__ void half_sweep(const Geom& geo, int c, const PhiloxPrefix& pre,
                                            const PhiloxKeys& key, Real* sp, int tid,
-                                           int tp, int K, const int4* units, Real J, Real hf, Real bp,
+                                           int tp, int K, const int4* units, const Couplings<Real>& cp,
                                            int& accepted, Partials<Real>& part) {
   const int S = geo.stride();
   const SpinView<Real> own(sp + c * 3 * S, S);
@@ -413,8 +559,7 @@ __device__ __forceinline__ void half_sweep(const Geom& geo, int c, const PhiloxP
             const V3<Real> cz = oth.ld(zn);
             const V3<Real> f =
                 add3(add3(add3(add3(add3(o0, oth.ld(nxo)), oth.ld(hh + oyp)), oth.ld(hh + oym)), cz), mz);
-            update<Real, kMeas, kEnergy>(static_cast<uint32_t>(2 * hh + p), pre, key, own, hh,
-                                         f.x, f.y, f.z, J, hf, bp, accepted, part);
+            update<kMeas, kEnergy>(static_cast<uint32_t>(2 * hh + p), pre, key, own, hh, f, cp, accepted, part);
             mz = o0;
             o0 = cz;
           }
@@ -435,7 +580,7 @@ __device__ __forceinline__ void half_sweep(const Geom& geo, int c, const PhiloxP
     int nn;
     const int i = geo.site(hh, c, nb, nn);
     attempt<Real, Geom::NNB, kMeas, kEnergy>(static_cast<uint32_t>(i), pre, key, own, oth,
-                                             hh, nb, nn, J, hf, bp, accepted, part);
+                                             hh, nb, nn, cp, accepted, part);
   }
 }
 
@@ -491,8 +636,25 @@ struct Meter {
   }
   // Store this warp's partials of the current measurement sweep and move to
   // the next (every lane calls, once per measurement sweep, in order).
-  __device__ void record(Partials<Real> part) {
-    using A = Arith<Real>;
+  // FP64 form: the warp's sums are exact integers; lane k < 4 rounds sum k.
+  __device__ void record(Partials<double> part) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      part.eb.add_lane(o);
+      part.mx.add_lane(o);
+      part.my.add_lane(o);
+      part.mz.add_lane(o);
+    }
+    const Wide v = lane == 0 ? part.eb : lane == 1 ? part.mx : lane == 2 ? part.my : part.mz;
+    const int64_t low = static_cast<int64_t>((static_cast<uint64_t>(v.w1) << 32) | v.w0);
+    const int32_t top = static_cast<int32_t>(v.w2) - static_cast<int32_t>(low >> 63);  // 0 if 64 bits hold it
+    double d = static_cast<double>(low);
+    if (__any_sync(0xffffffffu, top != 0)) d = fma(static_cast<double>(top), 0x1p64, d);
+    if (lane < 4) (cur_slot() + (slot_off + warp) * kRedSlots)[lane] = d * (lane == 0 ? kEnergyUnit : kSpinUnit);
+    advance();
+  }
+  __device__ void record(Partials<float> part) {
+    using A = Arith<float>;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       part.eb += A::shfl(part.eb, o);
@@ -605,20 +767,21 @@ struct Meter {
 // Initial spin of site i: uniform on the sphere (Sec. 2.2), uniform angles,
 // or the ordered start of Sec. 5.
 template <typename Real>
-__device__ __forceinline__ void initial_spin(uint32_t i, uint32_t c2, uint32_t c3i,
-                                             const SweepParams& P, int mode, Real& x, Real& y,
-                                             Real& z) {
-  using A = Arith<Real>;
+__device__ __forceinline__ V3<Real> initial_spin(uint32_t i, uint32_t c2, uint32_t c3i, const SweepParams& P,
+                                                 int mode) {
+  using S = Stored<Real>;
   const Philox4 r = philox4x32_10(i, 0u, c2, c3i, P.key);
-  if (mode == MP_INIT_ORDERED) {
-    x = Real(0);
-    y = Real(0);
-    z = Real(1);
-  } else if (mode == MP_INIT_ANGLES) {
-    A::init_angles(r.x, r.y, x, y, z);
-  } else {
-    A::trial(r.x, r.y, x, y, z);
+  if (mode == MP_INIT_ORDERED) return V3<Real>{S::from(Real(0)), S::from(Real(0)), S::from(Real(1))};
+  if (mode == MP_INIT_SPHERE) {
+    if constexpr (sizeof(Real) == 8) {
+      const Fix3 t = fix_trial(r.x, r.y, fix_root(r.x), sine_shared());
+      return V3<Real>{t.x, t.y, t.z};
+    }
   }
+  Real x, y, z;
+  if (mode == MP_INIT_ANGLES) Arith<Real>::init_angles(r.x, r.y, x, y, z);
+  else Arith<Real>::trial(r.x, r.y, x, y, z);
+  return V3<Real>{S::from(x), S::from(y), S::from(z)};
 }
 
 // --------------------------------------------------------- resumable state --
@@ -652,7 +815,7 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
   const uint32_t c3i = kTagInit | (static_cast<uint32_t>(sys_idx) << 8);
   const int init = path_init_mode(P.init_mode, path, sy.n_paths);
   const Real J = static_cast<Real>(sy.J), hf = static_cast<Real>(sy.h);
-  const Real bp = A::beta_param(sy.beta);
+  const Couplings<Real> cp(P.systems + sys_idx);
   // column segments per column (column_segments; 0 = decode every site: open
   // chains), and the host's table of the column-walk units when it was made
   // for this chunk (the table's K is then that of the same rule)
@@ -678,11 +841,12 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
   meter.start();
   unsigned char* st = path_state(P, sys_idx, path);
   Real* st_spins = st ? reinterpret_cast<Real*>(st + kStateHeader) : nullptr;
+  typename Stored<Real>::C* raw = reinterpret_cast<typename Stored<Real>::C*>(sp);
   __shared__ int cancel_flag[kMaxGroups];
   const int gidx = bar - 1;
 
   if (P.resume && st) {  // continue from the saved state
-    for (int k = tid; k < 6 * S; k += tp) sp[k] = st_spins[k];
+    for (int k = tid; k < 6 * S; k += tp) raw[k] = Stored<Real>::from(st_spins[k]);
     if (tid < kAccDoubles) meter.acc[tid] = reinterpret_cast<const double*>(st)[tid];
   } else {
     for (int c = 0; c < 2; ++c) {
@@ -692,9 +856,8 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
         int nb[Geom::NNB];
         int nn;
         const int i = geo.site(hh, c, nb, nn);
-        Real x, y, z;
-        initial_spin<Real>(static_cast<uint32_t>(i), c2, c3i, P, init, x, y, z);
-        own.st(hh, x, y, z);
+        const V3<Real> v = initial_spin<Real>(static_cast<uint32_t>(i), c2, c3i, P, init);
+        own.st(hh, v.x, v.y, v.z);
       }
     }
     if (tid < kAccDoubles) meter.acc[tid] = 0.0;
@@ -709,34 +872,30 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
   for (int64_t s = P.s_begin; s < P.s_end; ++s) {
     const uint32_t sw = static_cast<uint32_t>(s);
     const PhiloxPrefix pre = philox_prefix(sw, c2, c3u, P.key);
-    Partials<Real> part{Real(0), Real(0), Real(0), Real(0)};
+    Partials<Real> part;
     poll_cancel(P, s, tid, &cancel_flag[gidx]);
     if (s < P.n_therm) {
-      half_sweep<Real, Geom, false, false>(geo, 0, pre, P.key, sp, tid, tp, K, units, J, hf,
-                                           bp, accepted, part);
+      half_sweep<Real, Geom, false, false>(geo, 0, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
       group_sync(tp, bar);
       if (cancel_flag[gidx]) {
         canceled = true;
         break;
       }
-      half_sweep<Real, Geom, false, false>(geo, 1, pre, P.key, sp, tid, tp, K, units, J, hf,
-                                           bp, accepted, part);
+      half_sweep<Real, Geom, false, false>(geo, 1, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
       group_sync(tp, bar);
       continue;
     }
     // Measurement sweep j.  Colour-0 sites keep their values during the
     // colour-1 pass, so the colour-1 local fields give every bond once.
     const int64_t j = s - P.n_therm;
-    half_sweep<Real, Geom, true, false>(geo, 0, pre, P.key, sp, tid, tp, K, units, J, hf, bp,
-                                        accepted, part);
+    half_sweep<Real, Geom, true, false>(geo, 0, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
     group_sync(tp, bar);
     if (cancel_flag[gidx]) {
       canceled = true;
       break;
     }
     meter.maybe_flush(j);
-    half_sweep<Real, Geom, true, true>(geo, 1, pre, P.key, sp, tid, tp, K, units, J, hf, bp,
-                                       accepted, part);
+    half_sweep<Real, Geom, true, true>(geo, 1, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
     meter.record(part);
     group_sync(tp, bar);
   }
@@ -753,11 +912,11 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
     const SpinView<Real> own(sp + c * 3 * S, S);
     for (int hh = tid; hh < geo.count(c); hh += tp) {
       const V3<Real> v = own.ld(hh);
-      worst = fmax(worst, fabs(sqrt(v.x * v.x + v.y * v.y + v.z * v.z) - Real(1)));
+      worst = fmax(worst, norm_error(v));
     }
   }
   if (P.save && st) {
-    for (int k = tid; k < 6 * S; k += tp) st_spins[k] = sp[k];
+    for (int k = tid; k < 6 * S; k += tp) st_spins[k] = Stored<Real>::real(raw[k]);
     if (tid < kAccDoubles) reinterpret_cast<double*>(st)[tid] = meter.acc[tid];
   }
   meter.write_record(P.records + (sy.rec_offset + path) * MP_NREC, accepted,
@@ -772,9 +931,9 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
         int nn;
         const int i = geo.site(hh, c, nb, nn);
         const V3<Real> v = own.ld(hh);
-        out[3 * i + 0] = v.x;
-        out[3 * i + 1] = v.y;
-        out[3 * i + 2] = v.z;
+        out[3 * i + 0] = Stored<Real>::real(v.x);
+        out[3 * i + 1] = Stored<Real>::real(v.y);
+        out[3 * i + 2] = Stored<Real>::real(v.z);
       }
     }
   }
@@ -836,7 +995,7 @@ constexpr int kPairChunk = 8;
 template <typename Real, int L, bool kMeas, bool kEnergy>
 __device__ __forceinline__ void half_sweep_pair(int c, int zbase, const PhiloxPrefix& pre,
                                                 const PhiloxKeys& key, Real* sp, Real* partner_sp,
-                                                int tid, int tp, Real J, Real hf, Real bp,
+                                                int tid, int tp, const Couplings<Real>& cp,
                                                 int& accepted, Partials<Real>& part) {
   using G = PairGeom<L>;
   constexpr int HL = G::HL, HP = G::HP, ZL = G::ZL, S = G::S;
@@ -868,8 +1027,8 @@ __device__ __forceinline__ void half_sweep_pair(int c, int zbase, const PhiloxPr
         const V3<Real> f =
             add3(add3(add3(add3(add3(o0, oth.ld(nxo)), oth.ld(hh + oyp)), oth.ld(hh + oym)), cz), mz);
         // site index x + L(y + L z_global) = 2 (col + HP z_global) + p
-        update<Real, kMeas, kEnergy>(static_cast<uint32_t>(2 * (hh + HP * (zbase - 1)) + p), pre, key,
-                                     own, hh, f.x, f.y, f.z, J, hf, bp, accepted, part);
+        update<kMeas, kEnergy>(static_cast<uint32_t>(2 * (hh + HP * (zbase - 1)) + p), pre, key, own, hh, f, cp,
+                               accepted, part);
         mz = o0;
         o0 = cz;
       }
@@ -903,7 +1062,7 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
   const uint32_t c3i = kTagInit | (static_cast<uint32_t>(sys_idx) << 8);
   const int init = path_init_mode(P.init_mode, path, sy.n_paths);
   const Real J = static_cast<Real>(sy.J), hf = static_cast<Real>(sy.h);
-  const Real bp = A::beta_param(sy.beta);
+  const Couplings<Real> cp(P.systems + sys_idx);
   const int64_t j_first = P.s_begin > P.n_therm ? P.s_begin - P.n_therm : 0;
   Real* red0 = reinterpret_cast<Real*>(slice + slice_red_offset());
   Meter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
@@ -926,18 +1085,10 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
       const int col = h % HP, zl = h / HP;
       const int zg = (zbase + zl - 1 + L) % L;
       const int hg = col + HP * zg;  // half index in the whole lattice
-      Real x, y, z;
-      if (resume) {
-        const SpinView<Real> saved(st_spins + c * 3 * NH, NH);
-        const V3<Real> v = saved.ld(hg);
-        x = v.x;
-        y = v.y;
-        z = v.z;
-      } else {
-        const int p = (col / HL + zg + c) & 1;
-        initial_spin<Real>(static_cast<uint32_t>(2 * hg + p), c2, c3i, P, init, x, y, z);
-      }
-      own.st(h, x, y, z);
+      const int p = (col / HL + zg + c) & 1;
+      const V3<Real> v = resume ? SpinView<Real>(st_spins + c * 3 * NH, NH).ld(hg)
+                                : initial_spin<Real>(static_cast<uint32_t>(2 * hg + p), c2, c3i, P, init);
+      own.st(h, v.x, v.y, v.z);
     }
   }
   if (tid < kAccDoubles) meter.acc[tid] = (resume && rank == 0) ? reinterpret_cast<const double*>(st)[tid] : 0.0;
@@ -950,7 +1101,7 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
   for (int64_t s = P.s_begin; s < P.s_end; ++s) {
     const uint32_t sw = static_cast<uint32_t>(s);
     const PhiloxPrefix pre = philox_prefix(sw, c2, c3u, P.key);
-    Partials<Real> part{Real(0), Real(0), Real(0), Real(0)};
+    Partials<Real> part;
     // rank 0 polls the host's flag and tells both CTAs, so that they stop together
     if (rank == 0 && tid == 0 && P.cancel != nullptr && ((s - P.s_begin) % kCancelPoll) == 0 &&
         *P.cancel != 0) {
@@ -960,11 +1111,9 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
     }
     const bool meas = s >= P.n_therm;
     if (meas)
-      half_sweep_pair<Real, L, true, false>(0, zbase, pre, P.key, sp, partner_sp, tid, tp, J, hf, bp,
-                                            accepted, part);
+      half_sweep_pair<Real, L, true, false>(0, zbase, pre, P.key, sp, partner_sp, tid, tp, cp, accepted, part);
     else
-      half_sweep_pair<Real, L, false, false>(0, zbase, pre, P.key, sp, partner_sp, tid, tp, J, hf, bp,
-                                             accepted, part);
+      half_sweep_pair<Real, L, false, false>(0, zbase, pre, P.key, sp, partner_sp, tid, tp, cp, accepted, part);
     cluster_sync_all();
     if (pair_cancel) {
       canceled = true;
@@ -972,12 +1121,10 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
     }
     if (meas) {
       if (rank == 0) meter.maybe_flush(s - P.n_therm);
-      half_sweep_pair<Real, L, true, true>(1, zbase, pre, P.key, sp, partner_sp, tid, tp, J, hf, bp,
-                                           accepted, part);
+      half_sweep_pair<Real, L, true, true>(1, zbase, pre, P.key, sp, partner_sp, tid, tp, cp, accepted, part);
       meter.record(part);
     } else {
-      half_sweep_pair<Real, L, false, false>(1, zbase, pre, P.key, sp, partner_sp, tid, tp, J, hf, bp,
-                                             accepted, part);
+      half_sweep_pair<Real, L, false, false>(1, zbase, pre, P.key, sp, partner_sp, tid, tp, cp, accepted, part);
     }
     cluster_sync_all();
   }
@@ -995,7 +1142,7 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
     const SpinView<Real> own(sp + c * 3 * S, S);
     for (int h = tid + HP; h < HP * (ZL + 1); h += tp) {
       const V3<Real> v = own.ld(h);
-      worst = fmax(worst, fabs(sqrt(v.x * v.x + v.y * v.y + v.z * v.z) - Real(1)));
+      worst = fmax(worst, norm_error(v));
       const int col = h % HP, zg = zbase + h / HP - 1;
       const int hg = col + HP * zg;
       if (P.save && st) SpinView<Real>(st_spins + c * 3 * NH, NH).st(hg, v.x, v.y, v.z);
@@ -1190,7 +1337,7 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   const uint32_t c3i = kTagInit | (static_cast<uint32_t>(sys_idx) << 8);
   const int init = path_init_mode(P.init_mode, path, sy.n_paths);
   const Real J = static_cast<Real>(sy.J), hf = static_cast<Real>(sy.h);
-  const Real bp = A::beta_param(sy.beta);
+  const Couplings<Real> cp(P.systems + sys_idx);
   const int64_t j_first = P.s_begin > P.n_therm ? P.s_begin - P.n_therm : 0;
   Meter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
                     reinterpret_cast<Real*>(slice + slice_red_offset()),
@@ -1208,12 +1355,21 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   for (int i = resume ? N : tid; i < N; i += tp) {
     const int x = i % L, y = (i / L) % L, z = i / (L * L);
     const int c = (x + y + z) & 1;
-    Real sx, sy_, sz;
-    initial_spin<Real>(static_cast<uint32_t>(i), c2, c3i, P, init, sx, sy_, sz);
+    const V3<Real> v = initial_spin<Real>(static_cast<uint32_t>(i), c2, c3i, P, init);
     Real* hpl = plane(z, c);
     const int hp = (x >> 1) + HL * y;
-    SpinView<Real>(hpl, HP).st(hp, sx, sy_, sz);
+    SpinView<Real>(hpl, HP).st(hp, v.x, v.y, v.z);
   }
+  // Between calls the state holds doubles: the FP64 form's integers while a
+  // call runs, each half-plane converted in place.
+  auto convert_state = [&](auto&& f) {
+    if constexpr (sizeof(Real) == 8) {
+      for (int k = tid; k < 2 * L * 3 * HP; k += tp) f(lat + static_cast<int64_t>(k / (3 * HP)) * hps + k % (3 * HP));
+    }
+  };
+  auto to_stored = [](Real* w) { *reinterpret_cast<typename Stored<Real>::C*>(w) = Stored<Real>::from(*w); };
+  auto to_real = [](Real* w) { *w = Stored<Real>::real(*reinterpret_cast<typename Stored<Real>::C*>(w)); };
+  if (resume) convert_state(to_stored);
   fence_async_global();
   if (tid < kAccDoubles) meter.acc[tid] = resume ? reinterpret_cast<const double*>(st)[tid] : 0.0;
   if (tid == 0) abort_flag[gidx] = 0;
@@ -1247,7 +1403,7 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
     const PhiloxPrefix pre = philox_prefix(sw, c2, c3u, P.key);
     const bool meas = s >= P.n_therm;
     const int64_t j = s - P.n_therm;
-    Partials<Real> part{Real(0), Real(0), Real(0), Real(0)};
+    Partials<Real> part;
     const int64_t sc = s - P.s_begin;  // sweeps since the mbarriers were initialised
     auto parity0 = [&](int q) {
       return static_cast<uint32_t>((sc * per_sweep(q & 3, 4) + q / 4) & 1);
@@ -1303,14 +1459,11 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
         const uint32_t i = static_cast<uint32_t>(2 * (hp + HP * z) + p);
         if (meas) {
           if (energy)
-            update<Real, true, true>(i, pre, P.key, own, hp, f.x, f.y, f.z, J, hf, bp,
-                                     accepted, part);
+            update<true, true>(i, pre, P.key, own, hp, f, cp, accepted, part);
           else
-            update<Real, true, false>(i, pre, P.key, own, hp, f.x, f.y, f.z, J, hf, bp,
-                                      accepted, part);
+            update<true, false>(i, pre, P.key, own, hp, f, cp, accepted, part);
         } else {
-          update<Real, false, false>(i, pre, P.key, own, hp, f.x, f.y, f.z, J, hf, bp,
-                                     accepted, part);
+          update<false, false>(i, pre, P.key, own, hp, f, cp, accepted, part);
         }
       };
       if constexpr (kFixedRows) {
@@ -1337,11 +1490,11 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
             const uint32_t i = static_cast<uint32_t>(2 * (hp + HP * z) + p);
             if (meas) {
               if (energy)
-                update<Real, true, true>(i, pre, P.key, own, hp, f.x, f.y, f.z, J, hf, bp, accepted, part);
+                update<true, true>(i, pre, P.key, own, hp, f, cp, accepted, part);
               else
-                update<Real, true, false>(i, pre, P.key, own, hp, f.x, f.y, f.z, J, hf, bp, accepted, part);
+                update<true, false>(i, pre, P.key, own, hp, f, cp, accepted, part);
             } else {
-              update<Real, false, false>(i, pre, P.key, own, hp, f.x, f.y, f.z, J, hf, bp, accepted, part);
+              update<false, false>(i, pre, P.key, own, hp, f, cp, accepted, part);
             }
           }
         }
@@ -1402,7 +1555,10 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
     for (int k = 0; k < kSlots; ++k) mbar_inval(mbar + k);
   }
   group_sync(tp, bar);
-  if (!ok) return;  // the error flag is set; the path's record is not written
+  if (!ok) {  // the error flag is set; the path's record is not written
+    if (st) convert_state(to_real);
+    return;
+  }
   const int64_t n_meas_done = P.s_end > P.n_therm ? P.s_end - P.n_therm : 0;
   meter.finish(n_meas_done);
   group_sync(tp, bar);
@@ -1412,14 +1568,17 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
     const int x = i % L, y = (i / L) % L, z = i / (L * L);
     const int hp = (x >> 1) + HL * y;
     const V3<Real> v = SpinView<Real>(plane(z, (x + y + z) & 1), HP).ld(hp);
-    const Real a = v.x, b = v.y, c = v.z;
-    worst = fmax(worst, fabs(sqrt(a * a + b * b + c * c) - Real(1)));
+    worst = fmax(worst, norm_error(v));
     if (P.spins != nullptr) {
       double* out = P.spins + P.spin_offset[sys_idx] + path * 3 * static_cast<int64_t>(N);
-      out[3 * i + 0] = a;
-      out[3 * i + 1] = b;
-      out[3 * i + 2] = c;
+      out[3 * i + 0] = Stored<Real>::real(v.x);
+      out[3 * i + 1] = Stored<Real>::real(v.y);
+      out[3 * i + 2] = Stored<Real>::real(v.z);
     }
+  }
+  if (st) {
+    group_sync(tp, bar);  // every spin has been read
+    convert_state(to_real);
   }
   if (P.save && st && tid < kAccDoubles) reinterpret_cast<double*>(st)[tid] = meter.acc[tid];
   meter.write_record(P.records + (sy.rec_offset + path) * MP_NREC, accepted,
@@ -1462,6 +1621,10 @@ __global__ void __launch_bounds__(CtaLimit<Real, kLattice>::value, 1)
     sweep_kernel(const SweepParams P) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int s_item;
+  if constexpr (sizeof(Real) == 8) {  // read after the first barrier below
+    for (int k = static_cast<int>(threadIdx.x); k < 256; k += static_cast<int>(blockDim.x))
+      sine_shared()[k] = kSineTable.s[k];
+  }
   if constexpr (kLattice == kMixedKernel && sizeof(Real) == 4) {
     // First the lattices held by two CTAs: the cluster takes one path at a
     // time from its own queue (rank 0 draws, both CTAs read), then each CTA
