@@ -569,7 +569,7 @@ def main():
             subs[name] = {"value": job_throughput(s_att, world, k_steps, s_ms), "unit": "attempts/s",
                           "steps": k_steps, "warmup": k_warm, "ms_per_step": s_ms / k_steps,
                           "config": {"workload": ws["text"], "plan": s_plan}, "roofline": s_roof,
-                          "clocks": st["clocks"], "gpu_launches": 2 * k_steps}
+                          "clocks": st["clocks"], "gpu_launches": 4 * k_steps}
 
     cpu = None
     if rank == 0 and not args.no_cpu_baseline:
@@ -599,7 +599,7 @@ def main():
                     "d2h_bytes_per_step": d2h_total,
                     "layout": ("autotuned once per process: each step's new handle takes the layout "
                                "measured at the first create")},
-            "gpu_launches": 2 * args.steps,
+            "gpu_launches": 4 * args.steps,
             "roofline": roof,
             "cpu_baseline": cpu,
             "clocks": t["clocks"],

@@ -18,6 +18,7 @@ struct ReduceParams {
   // MP_R_MAX_PATHS paths: 2 n_paths doubles at 2 rec_offset per system
   // (nullptr when no system is that large).
   double* sort_buf;
+  double* work;  // scratch of the reduction's passes, reduce_work_doubles() doubles
 };
 
 struct BackwardParams {
@@ -69,6 +70,7 @@ cudaError_t launch_random_site(int precision, const SweepParams& p, int n_system
                                void* lattice, int64_t elements, cudaStream_t st);
 
 cudaError_t reduce_prepare();  // raise the dynamic shared memory limit
+int64_t reduce_work_doubles(int64_t total_paths, int n_systems);
 cudaError_t launch_reduce(const ReduceParams& p, int n_systems, int64_t max_paths, cudaStream_t st);
 cudaError_t launch_backward(const BackwardParams& p, int n_systems, cudaStream_t st);
 cudaError_t launch_philox(const uint32_t* ctr, int64_t n, uint64_t seed, uint32_t* out,

@@ -169,6 +169,7 @@ struct mp_state {
   int4* d_units = nullptr;         // column-walk unit tables (column_unit), one per (L, K, U)
   int64_t units_capacity = 0;      // entries allocated at d_units
   int64_t upload_bytes = 0;        // bytes the last upload_tables copied to the device
+  double* d_work = nullptr;        // scratch of the reduction
   double* d_sort = nullptr;        // sort space of the distribution coefficient (systems > 16384 paths)
   int* d_error = nullptr;          // nonzero when a bounded wait in a kernel gave up
   void* d_lattice = nullptr;       // HBM lattices of streamed paths
@@ -662,6 +663,7 @@ int enqueue_run(mp_state* h, int64_t s_begin, int64_t s_end, bool resume, bool s
   r.n_therm = std::min(s_end, h->n_therm);
   r.n_meas = std::max<int64_t>(0, s_end - h->n_therm);
   r.sort_buf = h->d_sort;
+  r.work = h->d_work;
   const unsigned evflag = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
   MP_CUDA(h, cudaMemsetAsync(h->d_queue, 0, 2 * sizeof(int), h->stream));
   MP_CUDA(h, cudaMemsetAsync(h->d_error, 0, sizeof(int), h->stream));
@@ -997,6 +999,7 @@ int mp_create_ex(const mp_config* cfg, mp_handle* out) {
   h->d_queue = static_cast<int*>(dev_alloc(h, 256));
   h->d_rec = static_cast<double*>(dev_alloc(h, sizeof(double) * MP_NREC * h->total_paths));
   h->d_est = static_cast<double*>(dev_alloc(h, sizeof(double) * MP_NEST * n));
+  h->d_work = static_cast<double*>(dev_alloc(h, sizeof(double) * reduce_work_doubles(h->total_paths, n)));
   h->d_spin_offset = static_cast<int64_t*>(dev_alloc(h, sizeof(int64_t) * n));
   h->d_thr = static_cast<unsigned long long*>(dev_alloc(h, sizeof(unsigned long long) * 10 * n));
   // unit tables: at most L^3/2 units per simple cubic size that fits shared memory
@@ -1004,8 +1007,8 @@ int mp_create_ex(const mp_config* cfg, mp_handle* out) {
   for (const mp_system& s : h->systems)
     if (s.lattice == MP_LATTICE_SC && s.L <= 26) h->units_capacity += static_cast<int64_t>(s.L) * s.L * s.L / 2;
   h->d_units = h->units_capacity > 0 ? static_cast<int4*>(dev_alloc(h, sizeof(int4) * h->units_capacity)) : nullptr;
-  if (!h->d_sys || !h->d_items || !h->d_queue || !h->d_rec || !h->d_est || !h->d_spin_offset ||
-      !h->d_thr || (h->units_capacity > 0 && !h->d_units))
+  if (!h->d_sys || !h->d_items || !h->d_queue || !h->d_rec || !h->d_est || !h->d_work ||
+      !h->d_spin_offset || !h->d_thr || (h->units_capacity > 0 && !h->d_units))
     return bail(fail(h, MP_ENOMEM, "device allocation failed"));
   h->d_error = static_cast<int*>(dev_alloc(h, 256));
   if (!h->d_error) return bail(fail(h, MP_ENOMEM, "device allocation failed"));
@@ -1370,13 +1373,16 @@ int mp_reduce(const mp_system* systems, int n_systems, int64_t n_therm, int64_t 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   DevSystem* d_sys = nullptr;
   double* d_sort = nullptr;
+  double* d_work = nullptr;
   auto done = [&](int code) {
     if (d_sys) cudaFree(d_sys);
+    if (d_work) cudaFree(d_work);
     if (d_sort) cudaFree(d_sort);
     cudaGetLastError();
     return code;
   };
   if (cudaMalloc(&d_sys, sizeof(DevSystem) * n_systems) != cudaSuccess ||
+      cudaMalloc(&d_work, sizeof(double) * reduce_work_doubles(rec, n_systems)) != cudaSuccess ||
       (max_paths > MP_R_MAX_PATHS && cudaMalloc(&d_sort, sizeof(double) * 2 * rec) != cudaSuccess))
     return done(fail(nullptr, MP_ENOMEM, "device allocation failed"));
   cudaError_t e = reduce_prepare();
@@ -1389,6 +1395,7 @@ int mp_reduce(const mp_system* systems, int n_systems, int64_t n_therm, int64_t 
   r.n_therm = n_therm;
   r.n_meas = n_meas;
   r.sort_buf = d_sort;
+  r.work = d_work;
   if (e == cudaSuccess) e = launch_reduce(r, n_systems, max_paths, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess)

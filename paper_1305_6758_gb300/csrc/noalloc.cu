@@ -11,7 +11,7 @@
 // pass from the sweep kernel to the reduction kernel, the work-queue counter,
 // and the device copies of the system, work-item and column-walk unit tables
 // -- in one file-scope __device__ array of fixed size.  Every GPU that loads
-// the library holds that array (about 3.4 MB) until the process exits.
+// the library holds that array (about 3.6 MB) until the process exits.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,6 +40,7 @@ constexpr int kMaxUnits = [] {
 
 struct NoallocScratch {
   double records[static_cast<size_t>(MP_NOALLOC_MAX_PATHS) * MP_NREC];
+  double work[MP_NOALLOC_MAX_PATHS + 64 * MP_NOALLOC_MAX_SYSTEMS];  // reduce_work_doubles of the limits
   WorkItem items[MP_NOALLOC_MAX_PATHS];
   DevSystem systems[MP_NOALLOC_MAX_SYSTEMS];
   int4 units[kMaxUnits];
@@ -200,6 +201,7 @@ extern "C" int mp_run_noalloc(const mp_system* systems, int n_systems, int preci
   r.est = d_estimates;
   r.n_therm = n_therm;
   r.n_meas = n_meas;
+  r.work = d->work;
   if (mpk::launch_sweep(precision, variant, p, grid, cta, smem, st) != cudaSuccess ||
       mpk::launch_reduce(r, n_systems, max_paths, st) != cudaSuccess) {
     cudaGetLastError();
