@@ -62,12 +62,18 @@ constexpr int kIsingThrBytes = 128;
 constexpr int ising_slice_spin_bytes(int L) { return kIsingThrBytes + 2 * (L / 2) * (L + 2); }
 
 // The random-site order (MP_FLAG_RANDOM_SITE, variant kRandomSiteKernel): one
-// thread per path, lattices in HBM (random_site_bytes_per_site bytes per site
-// and path).
+// warp per path (one thread for many paths of very few sites), lattices in shared
+// memory, or in HBM
+// (random_site_bytes_per_site bytes per site and path).
 constexpr int kRandomSiteKernel = -4;
+struct RandomSitePlan {
+  bool shared = false, thread_per_path = false;
+  int slice = 0, cta = 0, smem = 0, grid = 0;  // shared-memory bytes per warp, launch shape
+};
 int random_site_bytes_per_site(int precision);
-cudaError_t launch_random_site(int precision, const SweepParams& p, int n_systems, int64_t total_paths,
-                               void* lattice, int64_t elements, cudaStream_t st);
+cudaError_t random_site_plan(int precision, int64_t max_sites, int64_t total_paths, int device, RandomSitePlan* plan);
+cudaError_t launch_random_site(int precision, const RandomSitePlan& plan, const SweepParams& p, int n_systems,
+                               int64_t total_paths, void* lattice, int64_t elements, cudaStream_t st);
 
 cudaError_t reduce_prepare();  // raise the dynamic shared memory limit
 int64_t reduce_work_doubles(int64_t total_paths, int n_systems);

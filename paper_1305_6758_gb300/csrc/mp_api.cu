@@ -157,6 +157,7 @@ struct mp_state {
 
   int cta = 0, grid = 0, smem = 0;
   int variant = 0;  // sweep kernel variant (see kernels.h)
+  RandomSitePlan random;  // launch shape of the random-site order
 
   DevSystem* d_sys = nullptr;
   WorkItem* d_items = nullptr;
@@ -576,8 +577,7 @@ int plan(mp_state* h, const mp_config* cfg) {
   return MP_OK;
 }
 
-// The random-site order: one thread per path (128-thread CTAs), every path's
-// lattice in HBM; no work items.
+// The random-site order: one warp per path; no work items.
 int plan_random_site(mp_state* h) {
   const int n = static_cast<int>(h->systems.size());
   h->variant = kRandomSiteKernel;
@@ -612,11 +612,13 @@ int plan_random_site(mp_state* h) {
   }
   h->total_paths = rec;
   h->total_spins = spins;
-  h->cta = 128;
-  h->smem = 0;
-  const int64_t grid = (rec + 127) / 128;
-  if (grid > 0x7fffffffLL) return fail(h, MP_EINVAL, "too many paths");
-  h->grid = static_cast<int>(grid);
+  if ((rec + 127) / 128 > 0x7fffffffLL) return fail(h, MP_EINVAL, "too many paths");
+  int64_t max_sites = 0;
+  for (const DevSystem& d : h->hsys) max_sites = std::max<int64_t>(max_sites, d.N);
+  MP_CUDA(h, random_site_plan(h->precision, max_sites, rec, h->device, &h->random));
+  h->cta = h->random.cta;
+  h->smem = h->random.smem;
+  h->grid = h->random.grid;
   h->lattice_groups = 0;
   h->lattice_stride = 0;
   MP_CUDA(h, reduce_prepare());
@@ -669,7 +671,7 @@ int enqueue_run(mp_state* h, int64_t s_begin, int64_t s_end, bool resume, bool s
   MP_CUDA(h, cudaMemsetAsync(h->d_error, 0, sizeof(int), h->stream));
   MP_CUDA(h, cudaEventRecordWithFlags(h->ev[0], h->stream, evflag));
   if (h->variant == kRandomSiteKernel)
-    MP_CUDA(h, launch_random_site(h->precision, p, static_cast<int>(h->hsys.size()), h->total_paths,
+    MP_CUDA(h, launch_random_site(h->precision, h->random, p, static_cast<int>(h->hsys.size()), h->total_paths,
                                   h->d_lattice, h->total_spins / 3, h->stream));
   else
     MP_CUDA(h, launch_sweep(h->precision, h->variant, p, h->grid, h->cta, h->smem, h->stream));
@@ -684,7 +686,8 @@ int enqueue_run(mp_state* h, int64_t s_begin, int64_t s_end, bool resume, bool s
 // The HBM lattice buffers of the current plan (streamed paths), grown on demand.
 int ensure_lattice(mp_state* h) {
   size_t need = 0;
-  if (h->variant == kRandomSiteKernel) {  // every path's lattice
+  if (h->variant == kRandomSiteKernel) {  // every path's lattice, unless shared memory holds it
+    if (h->random.shared) return MP_OK;
     need = static_cast<size_t>(h->total_spins / 3) * random_site_bytes_per_site(h->precision);
   } else {
     if (h->lattice_groups == 0) return MP_OK;

@@ -245,10 +245,21 @@ struct Wide {
     const uint32_t hi = static_cast<uint32_t>(static_cast<uint64_t>(v) >> 32);
     add(static_cast<uint32_t>(v), hi, static_cast<uint32_t>(static_cast<int32_t>(hi) >> 31));
   }
-  __device__ __forceinline__ void add_lane(int o) {  // a butterfly step over the warp
-    const uint32_t a = __shfl_xor_sync(0xffffffffu, w0, o), b = __shfl_xor_sync(0xffffffffu, w1, o),
-                   c = __shfl_xor_sync(0xffffffffu, w2, o);
-    add(a, b, c);
+  __device__ __forceinline__ void add_warp() {  // every lane gets the warp's sum
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const uint32_t a = __shfl_xor_sync(0xffffffffu, w0, o), b = __shfl_xor_sync(0xffffffffu, w1, o),
+                     c = __shfl_xor_sync(0xffffffffu, w2, o);
+      add(a, b, c);
+    }
+  }
+  // The value as a double.
+  __device__ __forceinline__ double real() const {
+    const int64_t low = static_cast<int64_t>((static_cast<uint64_t>(w1) << 32) | w0);
+    const int32_t top = static_cast<int32_t>(w2) - static_cast<int32_t>(low >> 63);  // 0 if 64 bits hold it
+    double d = static_cast<double>(low);
+    if (top != 0) d = fma(static_cast<double>(top), 0x1p64, d);
+    return d;
   }
 };
 
@@ -416,12 +427,11 @@ static __device__ __noinline__ bool accept_exact(int64_t dx, int64_t dy, int64_t
 // moves; those take accept_exact), and the trial spin is evaluated to 2^-53 in
 // integers (fix_trial), by warps in which a move was accepted.  L = 16, three
 // temperatures of 1024 paths: 5.2e9 attempts/s with FP64 arithmetic, 5.5e10 so.
-template <bool kMeas, bool kEnergy>
-__device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
-                                       const SpinView<double>& own, int hh, V3<double> f,
-                                       const Couplings<double>& cp, int& accepted, Partials<double>& part) {
-  const Philox4 r = philox4x32_10(i, pre, key);
-  const V3<double> a = own.ld(hh);
+//
+// The accept test of the move drawn by r at the spin a in the local field f;
+// when it is accepted, n is the trial spin.
+__device__ __forceinline__ bool accept_fixed(const Philox4& r, V3<double> a, V3<double> f,
+                                             const Couplings<double>& cp, V3<double>& n) {
   const FixRoot q = fix_root(r.x);
   // d and h in units of 2^-28, as floats
   auto f28 = [](int64_t v) { return static_cast<float>(static_cast<int32_t>(v >> 25)); };
@@ -437,23 +447,37 @@ __device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, cons
   const float u = fmaf(static_cast<float>(r.z), 0x1p-32f, 0x1p-33f);
   bool ok = u < p * cp.lo;
   const bool open = !ok && !(u > p * cp.hi);  // undecided (NaN and infinity included)
-  V3<double> n = a;
   if (ok || open) {
     const Fix3 t = fix_trial(r.x, r.y, q, sine_shared());
     if (open) ok = accept_exact(t.x - a.x, t.y - a.y, t.z - a.z, f.x, f.y, f.z, cp.sys, r.z);
-    if (ok) {
-      own.st(hh, t.x, t.y, t.z);
-      n = V3<double>{t.x, t.y, t.z};
-      ++accepted;
-    }
+    n = V3<double>{t.x, t.y, t.z};
+  }
+  return ok;
+}
+
+// S . h in units of 2^-57, from (S 2^62) (h 2^59) 2^-64.
+__device__ __forceinline__ int64_t spin_dot(V3<double> s, V3<double> h) {
+  return __mul64hi(s.x << 9, h.x << 6) + __mul64hi(s.y << 9, h.y << 6) + __mul64hi(s.z << 9, h.z << 6);
+}
+
+template <bool kMeas, bool kEnergy>
+__device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
+                                       const SpinView<double>& own, int hh, V3<double> f,
+                                       const Couplings<double>& cp, int& accepted, Partials<double>& part) {
+  const Philox4 r = philox4x32_10(i, pre, key);
+  const V3<double> a = own.ld(hh);
+  V3<double> n;
+  if (accept_fixed(r, a, f, cp, n)) {
+    own.st(hh, n.x, n.y, n.z);
+    ++accepted;
+  } else {
+    n = a;
   }
   if (kMeas) {
     part.mx.add(n.x);
     part.my.add(n.y);
     part.mz.add(n.z);
-    // S . h in units of 2^-57: (S 2^62) (h 2^59) 2^-64
-    if (kEnergy)
-      part.eb.add(__mul64hi(n.x << 9, f.x << 6) + __mul64hi(n.y << 9, f.y << 6) + __mul64hi(n.z << 9, f.z << 6));
+    if (kEnergy) part.eb.add(spin_dot(n, f));
   }
 }
 
@@ -638,18 +662,11 @@ struct Meter {
   // the next (every lane calls, once per measurement sweep, in order).
   // FP64 form: the warp's sums are exact integers; lane k < 4 rounds sum k.
   __device__ void record(Partials<double> part) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      part.eb.add_lane(o);
-      part.mx.add_lane(o);
-      part.my.add_lane(o);
-      part.mz.add_lane(o);
-    }
-    const Wide v = lane == 0 ? part.eb : lane == 1 ? part.mx : lane == 2 ? part.my : part.mz;
-    const int64_t low = static_cast<int64_t>((static_cast<uint64_t>(v.w1) << 32) | v.w0);
-    const int32_t top = static_cast<int32_t>(v.w2) - static_cast<int32_t>(low >> 63);  // 0 if 64 bits hold it
-    double d = static_cast<double>(low);
-    if (__any_sync(0xffffffffu, top != 0)) d = fma(static_cast<double>(top), 0x1p64, d);
+    part.eb.add_warp();
+    part.mx.add_warp();
+    part.my.add_warp();
+    part.mz.add_warp();
+    const double d = (lane == 0 ? part.eb : lane == 1 ? part.mx : lane == 2 ? part.my : part.mz).real();
     if (lane < 4) (cur_slot() + (slot_off + warp) * kRedSlots)[lane] = d * (lane == 0 ? kEnergyUnit : kSpinUnit);
     advance();
   }
