@@ -41,12 +41,12 @@ bool sweep_supports_L(int precision, int L) {
 }
 cudaError_t sweep_prepare(int precision, int variant, int device, int* max_dynamic,
                           int* max_threads) {
-  if (is_ising_variant(variant)) return ising_prepare(variant, device, max_dynamic, max_threads);
+  if (variant == kIsingKernel) return ising_prepare(device, max_dynamic, max_threads);
   return precision == MP_FP64 ? sweep_prepare_fp64(variant, device, max_dynamic, max_threads)
                               : sweep_prepare_fp32(variant, device, max_dynamic, max_threads);
 }
 cudaError_t sweep_occupancy(int precision, int variant, int cta, int smem, int* blocks) {
-  if (is_ising_variant(variant)) return ising_occupancy(variant, cta, smem, blocks);
+  if (variant == kIsingKernel) return ising_occupancy(cta, smem, blocks);
   return precision == MP_FP64 ? sweep_occupancy_fp64(variant, cta, smem, blocks)
                               : sweep_occupancy_fp32(variant, cta, smem, blocks);
 }
@@ -56,7 +56,7 @@ cudaError_t sweep_cluster_occupancy(int precision, int variant, int cta, int sme
 }
 cudaError_t launch_sweep(int precision, int variant, const SweepParams& p, int grid, int cta,
                          int smem, cudaStream_t st) {
-  if (is_ising_variant(variant)) return launch_ising(variant, p, grid, cta, smem, st);
+  if (variant == kIsingKernel) return launch_ising(p, grid, cta, smem, st);
   return precision == MP_FP64 ? launch_sweep_fp64(variant, p, grid, cta, smem, st)
                               : launch_sweep_fp32(variant, p, grid, cta, smem, st);
 }
@@ -74,10 +74,11 @@ int64_t sites_of(const mp_system& s) {
   return s.lattice == MP_LATTICE_SC ? static_cast<int64_t>(s.L) * s.L * s.L : s.L;
 }
 
-// Shared-memory bytes of one path's spins (both colours) in the sweep kernels.
+// Bytes of one path's spins (both colours) in the sweep kernels' shared memory
+// and in saved states (Ising: in saved states, a byte per spin).
 int64_t lattice_bytes(const mp_system& s, int real) {
   const int64_t NH = (sites_of(s) + 1) / 2;
-  if (s.lattice == MP_LATTICE_ISING) return kIsingThrBytes + 2 * NH;
+  if (s.lattice == MP_LATTICE_ISING) return 128 + 2 * NH;
   return 6 * ((NH + 1) & ~int64_t{1}) * real;  // per colour: (x, y) pairs then z, even length
 }
 
@@ -343,7 +344,7 @@ int plan(mp_state* h, const mp_config* cfg) {
   auto global = [&](const mp_system& sy) { return in_place(sy, h->precision, h->flags, optin); };
   // lattices held by two-CTA clusters run in the mixed-size kernel
   auto variant_of = [&](const mp_system& sy) {
-    if (sy.lattice == MP_LATTICE_ISING) return ising_compiled_L(sy.L) ? ising_variant(sy.L) : kIsingKernel;
+    if (sy.lattice == MP_LATTICE_ISING) return kIsingKernel;
     if (sy.lattice == MP_LATTICE_CHAIN) return -1;
     if (paired(sy, h->precision, h->flags)) return 0;  // the mixed-size kernel
     if (!streamed(sy, h->precision, h->flags)) return sy.L;
@@ -360,8 +361,6 @@ int plan(mp_state* h, const mp_config* cfg) {
   }
   // streamed sizes mixed, or streamed with in-place ones: the streamed kernel runs both
   if (variant == 0 && all_streamed) variant = -2;
-  // Ising sizes mixed (batches are all Ising or all Heisenberg): the kernel for any L
-  if (variant == 0 && h->systems[0].lattice == MP_LATTICE_ISING) variant = kIsingKernel;
   h->variant = variant;
   int sms = 0, smem_max = 0, cta_max = 0;
   MP_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
@@ -390,6 +389,8 @@ int plan(mp_state* h, const mp_config* cfg) {
     sl = best_sl;
   };
   int max_tp = 32;
+  int64_t batch_paths = 0;
+  for (const mp_system& sy : h->systems) batch_paths += sy.n_paths;
   for (int k = 0; k < n; ++k) {
     const int64_t N = sites_of(h->systems[k]);
     const int NH = static_cast<int>((N + 1) / 2);
@@ -441,6 +442,8 @@ int plan(mp_state* h, const mp_config* cfg) {
       max_tp = std::max(max_tp, t);
       continue;
     }
+    if (t == 0 && h->systems[k].lattice == MP_LATTICE_ISING)
+      t = ising_threads(h->systems[k].L, (batch_paths + sms - 1) / sms, smem_max, 16);
     if (t == 0 && h->systems[k].lattice == MP_LATTICE_SC) {
       // a divisor of the sites per colour lets each thread walk a block of
       // columns; pick the one closest to the target sites per thread
@@ -460,7 +463,7 @@ int plan(mp_state* h, const mp_config* cfg) {
     tp[k] = t;
     // partial-sum ring: the largest power of two up to 16 sweeps that fits
     ring[k] = 16;
-    // shared-memory bytes of the lattice (Ising: with a copy of each boundary row)
+    // shared-memory bytes of the lattice
     const int64_t lat = h->systems[k].lattice == MP_LATTICE_ISING ? ising_slice_spin_bytes(h->systems[k].L)
                                                                    : lattice_bytes(h->systems[k], real);
     pick_ring(ring[k], slice[k], [&]() {
@@ -492,6 +495,10 @@ int plan(mp_state* h, const mp_config* cfg) {
   if (cta == 0) {
     cta = cta_max;
     while (cta / 2 >= std::max(max_tp, 128) && count_items(cta) < 2LL * sms) cta /= 2;
+    // Ising paths all take equally long, so the last round of a launch is
+    // partly empty: small CTAs spread its paths over every SM (four to an SM,
+    // each with 16 of its 64 named barriers)
+    if (variant == kIsingKernel) cta = std::max(max_tp, 256);
   }
   if (cta < max_tp) return fail(h, MP_EINVAL, "cta_threads %d below threads per path %d", cta, max_tp);
 
