@@ -118,7 +118,8 @@ struct Attempt<float> {
   __device__ __forceinline__ explicit Attempt(const Philox4& r) : r2(r.z) { Arith<float>::trial(r.x, r.y, tx, ty, tz); }
   __device__ __forceinline__ bool test(V3<float> a, V3<float> f, const Couplings<float>& cp, V3<float>& n) const {
     n = V3<float>{tx, ty, tz};
-    return Arith<float>::accept_move(tx - a.x, ty - a.y, tz - a.z, f.x, f.y, f.z, cp.J, cp.hf, cp.bp, r2);
+    using A = Arith<float>;
+    return A::accept_move(A::sub(tx, a.x), A::sub(ty, a.y), A::sub(tz, a.z), f.x, f.y, f.z, cp.J, cp.hf, cp.bp, r2);
   }
 };
 template <>
@@ -126,7 +127,12 @@ struct Attempt<double> {
   Philox4 r;
   __device__ __forceinline__ explicit Attempt(const Philox4& r_) : r(r_) {}
   __device__ __forceinline__ bool test(V3<double> a, V3<double> f, const Couplings<double>& cp, V3<double>& n) const {
-    return accept_fixed(r, a, f, cp, n);
+    bool ok = false;
+    move_fixed(r, a, f, cp, [&](V3<double> t) {
+      n = t;
+      ok = true;
+    });
+    return ok;
   }
 };
 

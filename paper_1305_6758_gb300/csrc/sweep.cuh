@@ -24,6 +24,7 @@
 // sites of one colour and their +-y, +-z neighbours are consecutive elements.
 #pragma once
 #include <cstdint>
+#include <type_traits>
 
 #include "common.cuh"
 #include "fixed64.cuh"
@@ -55,8 +56,8 @@ struct Arith<float> {
     // phi - pi = 2 pi (u1 - 1/2) lies in (-pi, pi), where the hardware sin/cos
     // are accurate; cos(phi) = -cos(phi - pi), sin(phi) = -sin(phi - pi).
     __sincosf(fmaf(6.28318531f, one_plus(r1), -9.42477763f), &s, &c);
-    x = -rad * c;
-    y = -rad * s;
+    x = __fmul_rn(-rad, c);
+    y = __fmul_rn(-rad, s);
   }
   static __device__ __forceinline__ void init_angles(uint32_t r0, uint32_t r1, float& x, float& y,
                                                      float& z) {
@@ -68,6 +69,19 @@ struct Arith<float> {
     z = ct;
   }
   static __device__ __forceinline__ float add(float a, float b) { return a + b; }
+  // a.b, every rounding spelled out: where a sum of products is left to the
+  // compiler, which product it rounds first changes with the code around it,
+  // and with it one accept decision in 1e8.
+  static __device__ __forceinline__ float dot(float ax, float ay, float az, float bx, float by, float bz) {
+    return __fmaf_rn(az, bz, __fmaf_rn(ax, bx, __fmul_rn(ay, by)));
+  }
+  static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+  static __device__ __forceinline__ float square(float x, float y, float z) {
+    return __fadd_rn(__fmaf_rn(y, y, __fmul_rn(x, x)), __fmul_rn(z, z));
+  }
+  static __device__ __forceinline__ float square_pair(float x, float y, float z) {
+    return __fadd_rn(__fmaf_rn(x, x, __fmul_rn(y, y)), __fmul_rn(z, z));
+  }
   // Metropolis test of the move S -> S + d in the local field (hx, hy, hz):
   // accept when dE <= 0, else iff u < exp(-beta dE) = 2^(-x), with
   // x = beta log2(e) dE = (-b J) d.h_loc + (-b h) d_z and b = beta log2(e)
@@ -75,7 +89,7 @@ struct Arith<float> {
   static __device__ __forceinline__ bool accept_move(float dx, float dy, float dz, float hx,
                                                      float hy, float hz, float J, float hf,
                                                      float blog2e, uint32_t r2) {
-    const float x = fmaf(-blog2e * J, dx * hx + dy * hy + dz * hz, (-blog2e * hf) * dz);
+    const float x = __fmaf_rn(__fmul_rn(-blog2e, J), dot(dx, dy, dz, hx, hy, hz), __fmul_rn(__fmul_rn(-blog2e, hf), dz));
     float p;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(-x));
     return x <= 0.0f || uni(r2) < p;
@@ -119,6 +133,9 @@ struct Arith<double> {
     z = ct;
   }
   static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
+  static __device__ __forceinline__ double square(double x, double y, double z) {
+    return fma(z, z, fma(y, y, x * x));
+  }
   static __device__ __forceinline__ double delta_e(double dx, double dy, double dz, double hx,
                                                    double hy, double hz, double J, double hf) {
     const double dot = __dadd_rn(__dadd_rn(__dmul_rn(dx, hx), __dmul_rn(dy, hy)), __dmul_rn(dz, hz));
@@ -384,18 +401,22 @@ struct Couplings<double> {
 // The Metropolis step at site i (half index hh of the colour view `own`)
 // given its local field f, Sec. 2.2: trial spin, energy change from the local
 // field, acceptance test.
+//
+// update_spin: the spin a held at the site is known; act = false (a thread
+// that walks along without a site) changes and counts nothing.  Returns the
+// spin the site has afterwards.
 template <bool kMeas, bool kEnergy>
-__device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
-                                       const SpinView<float>& own, int hh, V3<float> f,
-                                       const Couplings<float>& cp, int& accepted, Partials<float>& part) {
+__device__ __forceinline__ V3<float> update_spin(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
+                                                 const SpinView<float>& own, int hh, V3<float> a, V3<float> f,
+                                                 const Couplings<float>& cp, bool act, int& accepted,
+                                                 Partials<float>& part) {
   using A = Arith<float>;
   const Philox4 r = philox4x32_10(i, pre, key);
   float tx, ty, tz;
   A::trial(r.x, r.y, tx, ty, tz);
-  const V3<float> a = own.ld(hh);
   const float ax = a.x, ay = a.y, az = a.z;
   float nx = ax, ny = ay, nz = az;
-  if (A::accept_move(tx - ax, ty - ay, tz - az, f.x, f.y, f.z, cp.J, cp.hf, cp.bp, r.z)) {
+  if (A::accept_move(A::sub(tx, ax), A::sub(ty, ay), A::sub(tz, az), f.x, f.y, f.z, cp.J, cp.hf, cp.bp, r.z) && act) {
     own.st(hh, tx, ty, tz);
     nx = tx;
     ny = ty;
@@ -403,11 +424,21 @@ __device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, cons
     ++accepted;
   }
   if (kMeas) {
-    part.mx += nx;
-    part.my += ny;
-    part.mz += nz;
-    if (kEnergy) part.eb += nx * f.x + ny * f.y + nz * f.z;
+    part.mx += act ? nx : 0.0f;
+    part.my += act ? ny : 0.0f;
+    part.mz += act ? nz : 0.0f;
+    if (kEnergy) {
+      const float b = A::dot(nx, ny, nz, f.x, f.y, f.z);
+      part.eb += act ? b : 0.0f;
+    }
   }
+  return V3<float>{nx, ny, nz};
+}
+template <bool kMeas, bool kEnergy>
+__device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
+                                       const SpinView<float>& own, int hh, V3<float> f,
+                                       const Couplings<float>& cp, int& accepted, Partials<float>& part) {
+  update_spin<kMeas, kEnergy>(i, pre, key, own, hh, own.ld(hh), f, cp, true, accepted, part);
 }
 
 // The accept test in FP64, for moves whose FP32 acceptance is too close to
@@ -426,12 +457,14 @@ static __device__ __noinline__ bool accept_exact(int64_t dx, int64_t dy, int64_t
 // lies outside the FP32 acceptance's error bound (all but about 1e-5 of the
 // moves; those take accept_exact), and the trial spin is evaluated to 2^-53 in
 // integers (fix_trial), by warps in which a move was accepted.  L = 16, three
-// temperatures of 1024 paths: 5.2e9 attempts/s with FP64 arithmetic, 5.5e10 so.
+// temperatures of 1024 paths: 5.2e9 attempts/s with FP64 arithmetic, 7.3e10 so.
 //
-// The accept test of the move drawn by r at the spin a in the local field f;
-// when it is accepted, n is the trial spin.
-__device__ __forceinline__ bool accept_fixed(const Philox4& r, V3<double> a, V3<double> f,
-                                             const Couplings<double>& cp, V3<double>& n) {
+// The move drawn by r at the spin a in the local field f: accepted(trial spin)
+// is called when it is accepted (within the branch that evaluates the trial
+// spin: a second branch on the outcome costs 15%).
+template <class F>
+__device__ __forceinline__ void move_fixed(const Philox4& r, V3<double> a, V3<double> f, const Couplings<double>& cp,
+                                           F&& accepted) {
   const FixRoot q = fix_root(r.x);
   // d and h in units of 2^-28, as floats
   auto f28 = [](int64_t v) { return static_cast<float>(static_cast<int32_t>(v >> 25)); };
@@ -450,9 +483,8 @@ __device__ __forceinline__ bool accept_fixed(const Philox4& r, V3<double> a, V3<
   if (ok || open) {
     const Fix3 t = fix_trial(r.x, r.y, q, sine_shared());
     if (open) ok = accept_exact(t.x - a.x, t.y - a.y, t.z - a.z, f.x, f.y, f.z, cp.sys, r.z);
-    n = V3<double>{t.x, t.y, t.z};
+    if (ok) accepted(V3<double>{t.x, t.y, t.z});
   }
-  return ok;
 }
 
 // S . h in units of 2^-57, from (S 2^62) (h 2^59) 2^-64.
@@ -466,13 +498,12 @@ __device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, cons
                                        const Couplings<double>& cp, int& accepted, Partials<double>& part) {
   const Philox4 r = philox4x32_10(i, pre, key);
   const V3<double> a = own.ld(hh);
-  V3<double> n;
-  if (accept_fixed(r, a, f, cp, n)) {
-    own.st(hh, n.x, n.y, n.z);
+  V3<double> n = a;
+  move_fixed(r, a, f, cp, [&](V3<double> t) {
+    own.st(hh, t.x, t.y, t.z);
+    n = t;
     ++accepted;
-  } else {
-    n = a;
-  }
+  });
   if (kMeas) {
     part.mx.add(n.x);
     part.my.add(n.y);
@@ -631,6 +662,7 @@ struct Meter {
   // when two CTAs of a cluster hold the lattice), and the first of them this
   // CTA's warps write (the partner CTA writes into the owner's ring)
   int nslot = 0, slot_off = 0;
+  bool pair_form = false;  // |m|^2 rounded as the two-CTA form's records have it
 
   __device__ void start() {
     if (nslot == 0) nslot = nwarps;
@@ -695,7 +727,9 @@ struct Meter {
     using A = Arith<Real>;
     Real e = Real(0), ex = Real(0), ey = Real(0), ez = Real(0);
     if (lane < n) observe(slot(j0 + lane), e, ex, ey, ez);
-    const Real m2 = ex * ex + ey * ey + ez * ez;
+    Real m2;
+    if constexpr (sizeof(Real) == 4) m2 = pair_form ? A::square_pair(ex, ey, ez) : A::square(ex, ey, ez);
+    else m2 = A::square(ex, ey, ez);
     const Real m = sqrt(m2);
     for (int k = warp; k <= MP_R_MMZ; k += nwarps) {
       Real v;
@@ -1087,6 +1121,7 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
                     sy.ring, tp >> 5, tid & 31, tid >> 5, tid,
                     1.0 / static_cast<double>(sy.N), J, hf, j_first};
   meter.nslot = 2 * (tp >> 5);
+  meter.pair_form = true;
   meter.slot_off = rank == 0 ? 0 : (tp >> 5);
   meter.start();
   unsigned char* st = path_state(P, sys_idx, path);
@@ -1338,11 +1373,6 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   uint64_t* mbar = reinterpret_cast<uint64_t*>(slice + slice_spin_offset(tp, sy.ring));
   uint32_t* issued = reinterpret_cast<uint32_t*>(mbar + kSlots);
   Real* buf = reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring) + 128);
-  // buffer of colour c, step index q (see above): 4 slots for colour 0, 5 for colour 1
-  auto c0buf = [&](int q) { return buf + (q & 3) * hps; };
-  auto c1buf = [&](int q) { return buf + (4 + (q + 1) % 5) * hps; };
-  auto c0bar = [&](int q) { return mbar + (q & 3); };
-  auto c1bar = [&](int q) { return mbar + 4 + (q + 1) % 5; };
   // a resumable run keeps the path's lattice in its state; otherwise the
   // group's own HBM buffer holds it for the run
   unsigned char* st = path_state(P, sys_idx, path);
@@ -1363,20 +1393,41 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   meter.start();
   __shared__ int abort_flag[kMaxGroups];  // per thread group: a bounded wait gave up, or canceled
   const int gidx = bar - 1;
-  const bool producer = tid == 0;
+  // Two threads move the half-planes, of different warps where there are two
+  // (a step's copies and waits are some hundred serial cycles that the warp's
+  // other work waits for): producer 0 colour 0, ring slots 0 .. 3, producer 1
+  // colour 1, slots 4 .. 8.
+  const int producer = tid == 0 ? 0 : tid == (tp > 32 ? 32 : 1) ? 1 : -1;
+  uint32_t phases = 0;  // a producer's next wait parity of each slot
   const bool resume = P.resume && st;
   const double accepted_before = resume ? reinterpret_cast<const double*>(st)[kAccDoubles] : 0.0;
 
+  // In-plane thread layout: column hx, rows y0, y0 + RS, ...
+  const int RS = kRS > 0 ? kRS : tp / HL;
+  const bool active = tid < HL * RS;
+  const int hx = active ? tid % HL : 0;
+  const int y0 = active ? tid / HL : L;
+  // f(half-plane, half index, site index) for this thread's sites, plane by plane
+  auto for_sites = [&](auto&& f) {
+    for (int z = 0; z < L; ++z) {
+      for (int c = 0; c < 2; ++c) {
+        Real* hpl = plane(z, c);
+#pragma unroll 4
+        for (int y = y0; y < L; y += RS) {
+          const int hp = hx + HL * y;
+          f(hpl, hp, 2 * (hp + HP * z) + ((y + z + c) & 1));
+        }
+      }
+    }
+  };
+
   // Initial state straight into HBM (generic stores), visible to the bulk copies.
   const int N = sy.N;
-  for (int i = resume ? N : tid; i < N; i += tp) {
-    const int x = i % L, y = (i / L) % L, z = i / (L * L);
-    const int c = (x + y + z) & 1;
-    const V3<Real> v = initial_spin<Real>(static_cast<uint32_t>(i), c2, c3i, P, init);
-    Real* hpl = plane(z, c);
-    const int hp = (x >> 1) + HL * y;
-    SpinView<Real>(hpl, HP).st(hp, v.x, v.y, v.z);
-  }
+  if (!resume)
+    for_sites([&](Real* hpl, int hp, int i) {
+      const V3<Real> v = initial_spin<Real>(static_cast<uint32_t>(i), c2, c3i, P, init);
+      SpinView<Real>(hpl, HP).st(hp, v.x, v.y, v.z);
+    });
   // Between calls the state holds doubles: the FP64 form's integers while a
   // call runs, each half-plane converted in place.
   auto convert_state = [&](auto&& f) {
@@ -1390,28 +1441,31 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   fence_async_global();
   if (tid < kAccDoubles) meter.acc[tid] = resume ? reinterpret_cast<const double*>(st)[tid] : 0.0;
   if (tid == 0) abort_flag[gidx] = 0;
-  if (producer) {
+  if (tid == 0) {
     for (int k = 0; k < kSlots; ++k) {
       mbar_init(mbar + k, 1);
       issued[k] = 0;
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  auto load = [&](Real* dst, const Real* src, int slot) {  // producer only
+  auto load = [&](const Real* src, int slot) {  // the slot's producer only
     ++issued[slot];
-    tma_load(dst, src, bytes, mbar + slot);
+    tma_load(buf + slot * hps, src, bytes, mbar + slot);
+  };
+  // every load is waited for once, in the order of the loads of its slot
+  auto wait_load = [&](int slot) {
+    if (!mbar_wait(mbar + slot, (phases >> slot) & 1u, P.error)) abort_flag[gidx] = 1;
+    phases ^= 1u << slot;
   };
   group_sync(tp, bar);
 
-  // In-plane thread layout: column hx, rows y0, y0 + RS, ...
-  const int RS = kRS > 0 ? kRS : tp / HL;
   constexpr bool kFixedRows = kL > 0 && kRS > 0 && kL % kRS == 0;
-  const bool active = tid < HL * RS;
-  const int hx = active ? tid % HL : 0;
-  const int y0 = active ? tid / HL : L;
-  // loads per sweep into each ring slot, for the mbarrier phase parity: slot
-  // j of a ring of n slots takes the shifted step indices j, j + n, ... <= L+1
-  auto per_sweep = [&](int j, int n) { return (L + 1 - j) / n + 1; };
+  // FP32 with three or four rows per thread (the planner's layouts): see phase
+  constexpr bool kFourRows = sizeof(Real) == 4 && kRS == 0;
+  const bool four_rows = 3 * RS <= L && L <= 4 * RS, fourth = y0 + 3 * RS < L;
+  const int hp0 = hx + HL * y0;
+  const int ym0 = y0 == 0 ? (L - 1) * HL : -HL;  // rows that may wrap in y: the first and the last
+  const int yp2 = y0 + 2 * RS == L - 1 ? -(L - 1) * HL : HL, yp3 = y0 + 3 * RS == L - 1 ? -(L - 1) * HL : HL;
   int accepted = 0;
   bool ok = true;
 
@@ -1421,35 +1475,21 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
     const bool meas = s >= P.n_therm;
     const int64_t j = s - P.n_therm;
     Partials<Real> part;
-    const int64_t sc = s - P.s_begin;  // sweeps since the mbarriers were initialised
-    auto parity0 = [&](int q) {
-      return static_cast<uint32_t>((sc * per_sweep(q & 3, 4) + q / 4) & 1);
-    };
-    auto parity1 = [&](int q) {
-      const int qq = q + 1;
-      return static_cast<uint32_t>((sc * per_sweep(qq % 5, 5) + qq / 5) & 1);
-    };
     // Buffers first used at step q: colour-0 index q, colour-1 index q+1 (at
-    // q = 0 also colour-1 indices -1 and 0).  Only the producer waits on their
+    // q = 0 also colour-1 indices -1 and 0).  Only the producers wait on their
     // mbarriers; the group barrier after the wait hands the data to everyone.
-    auto wait_step = [&](int q) {
-      bool w = mbar_wait(c0bar(q), parity0(q), P.error);
-      if (q == 0) {
-        w = w && mbar_wait(c1bar(-1), parity1(-1), P.error);
-        w = w && mbar_wait(c1bar(0), parity1(0), P.error);
-      }
-      if (q < L) w = w && mbar_wait(c1bar(q + 1), parity1(q + 1), P.error);
-      if (!w) abort_flag[gidx] = 1;
-    };
     int cancel = 0;
     poll_cancel(P, s, tid, &cancel);
-    if (producer && cancel) abort_flag[gidx] = 1;  // stop before any copy of this sweep
-    if (producer && !cancel) {
-      tma_wait_all();  // the previous sweep's write-backs are complete
-      if (!(P.test_stall && s == P.s_begin)) load(c0buf(0), plane(0, 0), 0);
-      load(c0buf(1), plane(1 % L, 0), 1);
-      for (int q1 = -1; q1 <= 2; ++q1) load(c1buf(q1), plane(wrap(q1), 1), 4 + (q1 + 1) % 5);
-      wait_step(0);
+    if (cancel) abort_flag[gidx] = 1;  // (thread 0) stop before the sweep's first update
+    if (producer == 0 && !cancel) {
+      tma_wait_all();  // the previous sweep's write-backs of this colour are complete
+      if (!(P.test_stall && s == P.s_begin)) load(plane(0, 0), 0);
+      load(plane(1, 0), 1);
+      wait_load(0);
+    } else if (producer == 1) {
+      tma_wait_all();
+      for (int q1 = -1; q1 <= 2; ++q1) load(plane(wrap(q1), 1), 4 + q1 + 1);
+      for (int k = 4; k <= 6; ++k) wait_load(k);
     }
     group_sync(tp, bar);
     if (abort_flag[gidx]) {
@@ -1492,28 +1532,54 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
           constexpr int kRows = kL / kRS;
           const int pz = (y0 + z + c) & 1;
           const int xoa = pz ? oxp1 : oxm0, xob = pz ? oxm0 : oxp1;
+          auto rows = [&](auto meas_c, auto energy_c) {
 #pragma unroll
-          for (int k = 0; k < kRows; ++k) {
-            const int y = y0 + k * kRS;
-            const bool flip = ((k * kRS) & 1) != 0;
-            const int p = flip ? pz ^ 1 : pz;
-            const int hp = hx + HL * y;
-            const int xo = hp + (flip ? xob : xoa);
-            const int yp = (k == kRows - 1 && y == L - 1) ? hp - (L - 1) * HL : hp + HL;
-            const int ym = (k == 0 && y == 0) ? hp + (L - 1) * HL : hp - HL;
-            // the two x neighbours in either order (a + b = b + a exactly)
-            const V3<Real> f = add3(add3(add3(add3(add3(same.ld(hp), same.ld(xo)), same.ld(yp)), same.ld(ym)),
-                                         up.ld(hp)), dn.ld(hp));
-            const uint32_t i = static_cast<uint32_t>(2 * (hp + HP * z) + p);
-            if (meas) {
-              if (energy)
-                update<true, true>(i, pre, P.key, own, hp, f, cp, accepted, part);
-              else
-                update<true, false>(i, pre, P.key, own, hp, f, cp, accepted, part);
-            } else {
-              update<false, false>(i, pre, P.key, own, hp, f, cp, accepted, part);
+            for (int k = 0; k < kRows; ++k) {
+              const int y = y0 + k * kRS;
+              const bool flip = ((k * kRS) & 1) != 0;
+              const int p = flip ? pz ^ 1 : pz;
+              const int hp = hx + HL * y;
+              const int xo = hp + (flip ? xob : xoa);
+              const int yp = (k == kRows - 1 && y == L - 1) ? hp - (L - 1) * HL : hp + HL;
+              const int ym = (k == 0 && y == 0) ? hp + (L - 1) * HL : hp - HL;
+              // the two x neighbours in either order (a + b = b + a exactly)
+              const V3<Real> f = add3(add3(add3(add3(add3(same.ld(hp), same.ld(xo)), same.ld(yp)), same.ld(ym)),
+                                           up.ld(hp)), dn.ld(hp));
+              const uint32_t i = static_cast<uint32_t>(2 * (hp + HP * z) + p);
+              update<decltype(meas_c)::value, decltype(energy_c)::value>(i, pre, P.key, own, hp, f, cp, accepted, part);
             }
-          }
+          };
+          // no branch between the rows: their Philox chains are interleaved
+          if (!meas) rows(std::false_type{}, std::false_type{});
+          else if (energy) rows(std::true_type{}, std::true_type{});
+          else rows(std::true_type{}, std::false_type{});
+        }
+      } else if (kFourRows && four_rows) {
+        if constexpr (kFourRows) {
+          if (!active) return;
+          // Rows y0 + k RS, k = 0 .. 3, the fourth only where it lies in the
+          // lattice (act): offsets, parities and wraps once per thread, no
+          // branch between the rows, whose Philox chains the compiler interleaves.
+          const int pz = (y0 + z + c) & 1;
+          const int xoa = pz ? oxp1 : oxm0, xob = pz ? oxm0 : oxp1;
+          const int xoc = (RS & 1) ? xob : xoa, pc = (RS & 1) ? pz ^ 1 : pz;
+          auto rows = [&](auto meas_c, auto energy_c) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const bool act = k < 3 || fourth;
+              const int hp = hp0 + (act ? k * (HL * RS) : 0);
+              const int xo = hp + (k & 1 ? xoc : xoa), p = k & 1 ? pc : pz;
+              const int yp = hp + (k == 3 ? yp3 : k == 2 ? yp2 : HL), ym = hp + (k == 0 ? ym0 : -HL);
+              const V3<Real> f = add3(add3(add3(add3(add3(same.ld(hp), same.ld(xo)), same.ld(yp)), same.ld(ym)),
+                                           up.ld(hp)), dn.ld(hp));
+              update_spin<decltype(meas_c)::value, decltype(energy_c)::value>(
+                  static_cast<uint32_t>(2 * (hp + HP * z) + p), pre, P.key, own, hp, own.ld(hp), f, cp, act, accepted,
+                  part);
+            }
+          };
+          if (!meas) rows(std::false_type{}, std::false_type{});
+          else if (energy) rows(std::true_type{}, std::true_type{});
+          else rows(std::true_type{}, std::false_type{});
         }
       } else {
 #pragma unroll 4
@@ -1526,32 +1592,49 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
     // own results of phase (a), and every other value either phase reads was
     // written before the previous barrier (in-plane neighbours of the other
     // colour come from the previous step) or is written after the next one.
+    // the buffers of colour-0 indices q-2, q-1, q and colour-1 indices q-1, q, q+1
+    Real *const end0 = buf + 4 * hps, *const end1 = buf + 9 * hps;
+    Real *p0m2 = buf + 2 * hps, *p0m1 = buf + 3 * hps, *p0 = buf;
+    Real *p1m1 = end0, *p1 = end0 + hps, *p1p1 = end0 + 2 * hps;
+    int next0 = 2, next1 = 4 + 4;  // slots of the loads issued after a step: colour-0 index q+2, colour-1 index q+3
     for (int q = 0; q <= L + 1; ++q) {
-      if (q < L) phase(0, q, c0buf(q), c1buf(q), c1buf(q + 1), c1buf(q - 1), false);
-      if (q >= 2) phase(1, wrap(q - 1), c1buf(q - 1), c0buf(q - 1), c0buf(q), c0buf(q - 2), meas);
+      if (q < L) phase(0, q, p0, p1, p1p1, p1m1, false);
+      if (q >= 2) phase(1, q > L ? 0 : q - 1, p1m1, p0m1, p0, p0m2, meas);
       fence_async_shared();
-      // the buffers step q+1 starts with were issued at step q-1: the producer
-      // confirms them now, and the barrier below hands them to every thread
-      if (producer && q + 1 <= L + 1) wait_step(q + 1);
+      // the buffers step q+1 starts with were issued at step q-1: their
+      // producer confirms them now, and the barrier below hands them to every
+      // thread
+      if (producer == 0 && q <= L) wait_load((q + 1) & 3);
+      if (producer == 1 && q + 1 < L) wait_load(next1 == 4 ? 8 : next1 - 1);  // colour-1 index q+2
       group_sync(tp, bar);
       if (abort_flag[gidx]) {
         ok = false;
         break;
       }
       if (meas && q == 0) meter.maybe_flush(j);
-      if (producer) {  // after the barrier: the buffers just written are complete
-        if (q < L) tma_store(plane(q, 0), c0buf(q), bytes);
-        if (q >= 2) tma_store(plane(wrap(q - 1), 1), c1buf(q - 1), bytes);
-        // the slots refilled now last held colour-0 index q-2 (stored after
-        // step q-2) and colour-1 index q-2 (stored after step q-1): all but
-        // this step's (at most two) store groups must have finished reading
-        // shared memory
-        tma_wait_read(2);
+      // After the barrier the buffers just written are complete.  The slot
+      // refilled now last held colour-0 index q-2 (stored after step q-2), or
+      // colour-1 index q-2 (stored after step q-1): all but this step's store
+      // must have finished reading shared memory.
+      if (producer == 0) {
+        if (q < L) tma_store(plane(q, 0), p0, bytes);
+        tma_wait_read(1);
         // colour-0 step indices L and L+1 reload planes 0 and 1 written this sweep
         if (q + 2 >= L) tma_wait_all();
-        if (q + 2 <= L + 1) load(c0buf(q + 2), plane(wrap(q + 2), 0), (q + 2) & 3);
-        if (q + 3 <= L) load(c1buf(q + 3), plane(wrap(q + 3), 1), 4 + (q + 4) % 5);
+        if (q + 2 <= L + 1) load(plane(q + 2 >= L ? q + 2 - L : q + 2, 0), next0);
+      } else if (producer == 1) {
+        if (q >= 2) tma_store(plane(q > L ? 0 : q - 1, 1), p1m1, bytes);
+        tma_wait_read(1);
+        if (q + 3 <= L) load(plane(q + 3 == L ? 0 : q + 3, 1), next1);
       }
+      next0 = (next0 + 1) & 3;
+      next1 = next1 == 8 ? 4 : next1 + 1;
+      p0m2 = p0m1;
+      p0m1 = p0;
+      p0 = p0 + hps == end0 ? buf : p0 + hps;
+      p1m1 = p1;
+      p1 = p1p1;
+      p1p1 = p1p1 + hps == end1 ? end0 : p1p1 + hps;
     }
     if (!ok) break;
     if (meas) {
@@ -1559,17 +1642,18 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
       group_sync(tp, bar);
     }
   }
-  if (producer) {
+  if (producer >= 0) {
+    const int k0 = producer == 0 ? 0 : 4, k1 = producer == 0 ? 4 : kSlots;
     if (!ok) {
       // a load did not arrive in time: wait (bounded) for every load still
       // in flight before the shared memory is given up
-      for (int k = 0; k < kSlots; ++k)
+      for (int k = k0; k < k1; ++k)
         if (issued[k] > 0) mbar_wait(mbar + k, (issued[k] - 1) & 1, P.error);
     }
     tma_wait_all();
     fence_async_global();
-    // every consumer passed its last wait before the last barrier
-    for (int k = 0; k < kSlots; ++k) mbar_inval(mbar + k);
+    // every wait on them was before the last barrier, or just above
+    for (int k = k0; k < k1; ++k) mbar_inval(mbar + k);
   }
   group_sync(tp, bar);
   if (!ok) {  // the error flag is set; the path's record is not written
@@ -1581,17 +1665,17 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   group_sync(tp, bar);
 
   Real worst = Real(0);  // in the working precision: FP64 runs at 1/64 rate on this GPU
-  for (int i = tid; i < N; i += tp) {
-    const int x = i % L, y = (i / L) % L, z = i / (L * L);
-    const int hp = (x >> 1) + HL * y;
-    const V3<Real> v = SpinView<Real>(plane(z, (x + y + z) & 1), HP).ld(hp);
-    worst = fmax(worst, norm_error(v));
-    if (P.spins != nullptr) {
-      double* out = P.spins + P.spin_offset[sys_idx] + path * 3 * static_cast<int64_t>(N);
+  if (P.spins == nullptr) {
+    for_sites([&](Real* hpl, int hp, int) { worst = fmax(worst, norm_error(SpinView<Real>(hpl, HP).ld(hp))); });
+  } else {
+    double* out = P.spins + P.spin_offset[sys_idx] + path * 3 * static_cast<int64_t>(N);
+    for_sites([&](Real* hpl, int hp, int i) {
+      const V3<Real> v = SpinView<Real>(hpl, HP).ld(hp);
+      worst = fmax(worst, norm_error(v));
       out[3 * i + 0] = Stored<Real>::real(v.x);
       out[3 * i + 1] = Stored<Real>::real(v.y);
       out[3 * i + 2] = Stored<Real>::real(v.z);
-    }
+    });
   }
   if (st) {
     group_sync(tp, bar);  // every spin has been read
