@@ -41,9 +41,10 @@ struct Arith;
 template <>
 struct Arith<float> {
   // 1 + m 2^-23 with m the top 23 bits of r, built from the bits (no int->float
-  // conversion); the uniform is that minus (1 - 2^-24) = (2m + 1) 2^-24, exactly.
+  // conversion; the sum is one shift-and-add instruction, an "or" would be
+  // two); the uniform is that minus (1 - 2^-24) = (2m + 1) 2^-24, exactly.
   static __device__ __forceinline__ float one_plus(uint32_t r) {
-    return __uint_as_float(0x3f800000u | (r >> 9));
+    return __uint_as_float(0x3f800000u + (r >> 9));
   }
   static __device__ __forceinline__ float uni(uint32_t r) { return one_plus(r) - 0.99999994f; }
   // Trial direction uniform on the sphere: cos(theta) = 2u0 - 1, phi = 2 pi u1.
@@ -85,14 +86,16 @@ struct Arith<float> {
   // Metropolis test of the move S -> S + d in the local field (hx, hy, hz):
   // accept when dE <= 0, else iff u < exp(-beta dE) = 2^(-x), with
   // x = beta log2(e) dE = (-b J) d.h_loc + (-b h) d_z and b = beta log2(e)
-  // precomputed per path (the two products are loop invariants).
+  // precomputed per path (the two products are loop invariants).  One compare
+  // decides both: 2^(-x) >= 1 > u for x <= 0 (the hardware's ex2 gives at least 1
+  // for every argument >= 0, checked over all floats).
   static __device__ __forceinline__ bool accept_move(float dx, float dy, float dz, float hx,
                                                      float hy, float hz, float J, float hf,
                                                      float blog2e, uint32_t r2) {
     const float x = __fmaf_rn(__fmul_rn(-blog2e, J), dot(dx, dy, dz, hx, hy, hz), __fmul_rn(__fmul_rn(-blog2e, hf), dz));
     float p;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(-x));
-    return x <= 0.0f || uni(r2) < p;
+    return uni(r2) < p;
   }
   static __device__ __forceinline__ float beta_param(double beta) {
     return static_cast<float>(beta * 1.4426950408889634);
