@@ -40,6 +40,8 @@ cudaError_t sweep_occupancy(int precision, int variant, int cta, int smem, int* 
 cudaError_t launch_sweep(int precision, int variant, const SweepParams& p, int grid, int cta,
                          int smem, cudaStream_t st);
 
+// Open chains only, each with at least as many threads as sites of a colour.
+constexpr int kChainOne = -6;
 // The streamed kernels compiled for simple cubic L = 32 and L = 64 (all
 // systems of the batch streamed at that size).
 constexpr int kStreamL32 = -1032;

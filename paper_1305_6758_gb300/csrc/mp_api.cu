@@ -495,6 +495,15 @@ int plan(mp_state* h, const mp_config* cfg) {
                   slice[k], smem_max);
     max_tp = std::max(max_tp, t);
   }
+  if (variant == -1) {  // chains with one site of a colour per thread have their own kernel
+    bool one = true;
+    for (int k = 0; k < n; ++k) one = one && (sites_of(h->systems[k]) + 1) / 2 <= tp[k];
+    if (one) {
+      int dyn = 0, threads = 0;
+      h->variant = variant = kChainOne;
+      MP_CUDA(h, sweep_prepare(h->precision, variant, h->device, &dyn, &threads));
+    }
+  }
   auto paths_per_cta = [&](int k, int cta) {
     if (paired(h->systems[k], h->precision, h->flags)) return 1;  // one path per cluster
     int g = cta / tp[k];

@@ -405,25 +405,21 @@ struct Couplings<double> {
 // given its local field f, Sec. 2.2: trial spin, energy change from the local
 // field, acceptance test.
 //
-// update_spin: the spin a held at the site is known; act = false (a thread
-// that walks along without a site) changes and counts nothing.  Returns the
-// spin the site has afterwards.
+// settle: the trial spin t and the spin a held at the site are known; act =
+// false (a thread that walks along without a site) changes and counts
+// nothing.
 template <bool kMeas, bool kEnergy>
-__device__ __forceinline__ V3<float> update_spin(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
-                                                 const SpinView<float>& own, int hh, V3<float> a, V3<float> f,
-                                                 const Couplings<float>& cp, bool act, int& accepted,
-                                                 Partials<float>& part) {
+__device__ __forceinline__ void settle(V3<float> t, uint32_t r2, const SpinView<float>& own, int hh, V3<float> a,
+                                       V3<float> f, const Couplings<float>& cp, bool act, int& accepted,
+                                       Partials<float>& part) {
   using A = Arith<float>;
-  const Philox4 r = philox4x32_10(i, pre, key);
-  float tx, ty, tz;
-  A::trial(r.x, r.y, tx, ty, tz);
-  const float ax = a.x, ay = a.y, az = a.z;
-  float nx = ax, ny = ay, nz = az;
-  if (A::accept_move(A::sub(tx, ax), A::sub(ty, ay), A::sub(tz, az), f.x, f.y, f.z, cp.J, cp.hf, cp.bp, r.z) && act) {
-    own.st(hh, tx, ty, tz);
-    nx = tx;
-    ny = ty;
-    nz = tz;
+  float nx = a.x, ny = a.y, nz = a.z;
+  if (A::accept_move(A::sub(t.x, a.x), A::sub(t.y, a.y), A::sub(t.z, a.z), f.x, f.y, f.z, cp.J, cp.hf, cp.bp, r2) &&
+      act) {
+    own.st(hh, t.x, t.y, t.z);
+    nx = t.x;
+    ny = t.y;
+    nz = t.z;
     ++accepted;
   }
   if (kMeas) {
@@ -435,7 +431,16 @@ __device__ __forceinline__ V3<float> update_spin(uint32_t i, const PhiloxPrefix&
       part.eb += act ? b : 0.0f;
     }
   }
-  return V3<float>{nx, ny, nz};
+}
+template <bool kMeas, bool kEnergy>
+__device__ __forceinline__ void update_spin(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
+                                            const SpinView<float>& own, int hh, V3<float> a, V3<float> f,
+                                            const Couplings<float>& cp, bool act, int& accepted,
+                                            Partials<float>& part) {
+  const Philox4 r = philox4x32_10(i, pre, key);
+  V3<float> t;
+  Arith<float>::trial(r.x, r.y, t.x, t.y, t.z);
+  settle<kMeas, kEnergy>(t, r.z, own, hh, a, f, cp, act, accepted, part);
 }
 template <bool kMeas, bool kEnergy>
 __device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, const PhiloxKeys& key,
@@ -462,6 +467,30 @@ static __device__ __noinline__ bool accept_exact(int64_t dx, int64_t dy, int64_t
 // integers (fix_trial), by warps in which a move was accepted.  L = 16, three
 // temperatures of 1024 paths: 5.2e9 attempts/s with FP64 arithmetic, 7.3e10 so.
 //
+// The FP32 stage of a move: the trial direction in units of 2^-28 and the uniform.
+struct FixDraw {
+  float tx, ty, tz, u;
+};
+__device__ __forceinline__ FixDraw fix_draw(const Philox4& r, const FixRoot& q) {
+  const float rad = q.nf * q.y * 0x1p-4f;  // sqrt(n) 2^-32 2^28
+  float s, c;
+  // phi - pi = (r1 + 1/2 - 2^31) 2 pi 2^-32; sine and cosine change sign
+  __sincosf(static_cast<float>(static_cast<int32_t>(r.y ^ 0x80000000u)) * 1.46291808e-9f, &s, &c);
+  return FixDraw{-rad * c, -rad * s, static_cast<float>(static_cast<int32_t>(r.x ^ 0x80000000u)) * 0.125f,
+                 fmaf(static_cast<float>(r.z), 0x1p-32f, 0x1p-33f)};
+}
+// Accepted for certain (ok), or undecided (open; NaN and infinity included).
+__device__ __forceinline__ void fix_test(const FixDraw& d, V3<double> a, V3<double> f, const Couplings<double>& cp,
+                                         bool& ok, bool& open) {
+  auto f28 = [](int64_t v) { return static_cast<float>(static_cast<int32_t>(v >> 25)); };
+  const float dx = d.tx - f28(a.x), dy = d.ty - f28(a.y), dz = d.tz - f28(a.z);
+  const float dot = dx * f28(f.x) + dy * f28(f.y) + dz * f28(f.z);
+  float p;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(fmaf(cp.cj, dot, cp.ch * dz)));
+  ok = d.u < p * cp.lo;
+  open = !ok && !(d.u > p * cp.hi);
+}
+
 // The move drawn by r at the spin a in the local field f: accepted(trial spin)
 // is called when it is accepted (within the branch that evaluates the trial
 // spin: a second branch on the outcome costs 15%).
@@ -469,20 +498,8 @@ template <class F>
 __device__ __forceinline__ void move_fixed(const Philox4& r, V3<double> a, V3<double> f, const Couplings<double>& cp,
                                            F&& accepted) {
   const FixRoot q = fix_root(r.x);
-  // d and h in units of 2^-28, as floats
-  auto f28 = [](int64_t v) { return static_cast<float>(static_cast<int32_t>(v >> 25)); };
-  const float rad = q.nf * q.y * 0x1p-4f;  // sqrt(n) 2^-32 2^28
-  float sp, cph;
-  // phi - pi = (r1 + 1/2 - 2^31) 2 pi 2^-32; sine and cosine change sign
-  __sincosf(static_cast<float>(static_cast<int32_t>(r.y ^ 0x80000000u)) * 1.46291808e-9f, &sp, &cph);
-  const float dx = -rad * cph - f28(a.x), dy = -rad * sp - f28(a.y);
-  const float dz = static_cast<float>(static_cast<int32_t>(r.x ^ 0x80000000u)) * 0.125f - f28(a.z);
-  const float dot = dx * f28(f.x) + dy * f28(f.y) + dz * f28(f.z);
-  float p;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(fmaf(cp.cj, dot, cp.ch * dz)));
-  const float u = fmaf(static_cast<float>(r.z), 0x1p-32f, 0x1p-33f);
-  bool ok = u < p * cp.lo;
-  const bool open = !ok && !(u > p * cp.hi);  // undecided (NaN and infinity included)
+  bool ok, open;
+  fix_test(fix_draw(r, q), a, f, cp, ok, open);
   if (ok || open) {
     const Fix3 t = fix_trial(r.x, r.y, q, sine_shared());
     if (open) ok = accept_exact(t.x - a.x, t.y - a.y, t.z - a.z, f.x, f.y, f.z, cp.sys, r.z);
@@ -514,6 +531,52 @@ __device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, cons
     if (kEnergy) part.eb.add(spin_dot(n, f));
   }
 }
+
+// One-site form (see run_path): a move drawn ahead of its update.
+template <typename Real>
+struct Ahead;
+template <>
+struct Ahead<float> {
+  V3<float> t;
+  uint32_t r2;
+  __device__ __forceinline__ explicit Ahead(const Philox4& r) : r2(r.z) { Arith<float>::trial(r.x, r.y, t.x, t.y, t.z); }
+  template <bool kMeas, bool kEnergy>
+  __device__ __forceinline__ void apply(const SpinView<float>& own, int hh, V3<float> f, const Couplings<float>& cp,
+                                        bool act, int& accepted, Partials<float>& part) const {
+    settle<kMeas, kEnergy>(t, r2, own, hh, own.ld(hh), f, cp, act, accepted, part);
+  }
+};
+template <>
+struct Ahead<double> {
+  FixDraw d;
+  Fix3 t;
+  uint32_t r2;
+  __device__ __forceinline__ explicit Ahead(const Philox4& r) : r2(r.z) {
+    const FixRoot q = fix_root(r.x);
+    d = fix_draw(r, q);
+    t = fix_trial(r.x, r.y, q, sine_shared());
+  }
+  template <bool kMeas, bool kEnergy>
+  __device__ __forceinline__ void apply(const SpinView<double>& own, int hh, V3<double> f, const Couplings<double>& cp,
+                                        bool act, int& accepted, Partials<double>& part) const {
+    const V3<double> a = own.ld(hh);
+    bool ok, open;
+    fix_test(d, a, f, cp, ok, open);
+    if (open) ok = accept_exact(t.x - a.x, t.y - a.y, t.z - a.z, f.x, f.y, f.z, cp.sys, r2);
+    ok = ok && act;
+    const V3<double> n = ok ? V3<double>{t.x, t.y, t.z} : a;
+    if (ok) {
+      own.st(hh, n.x, n.y, n.z);
+      ++accepted;
+    }
+    if (kMeas && act) {
+      part.mx.add(n.x);
+      part.my.add(n.y);
+      part.mz.add(n.z);
+      if (kEnergy) part.eb.add(spin_dot(n, f));
+    }
+  }
+};
 
 // One Metropolis attempt with the neighbours' half indices nb[0..nn) in `oth`,
 // summed in the fixed order nb[0], nb[1], ...
@@ -857,7 +920,15 @@ __device__ __forceinline__ void poll_cancel(const SweepParams& P, int64_t s, int
 // ------------------------------------------------------------- one path --
 // The lattice lives in the slice's shared memory, or in HBM at `hbm_spins`
 // (the same layout) when it is updated in place there.
-template <typename Real, class Geom>
+//
+// kOne: every thread owns at most one site of each colour (tp >= sites per
+// colour: short chains, L <= 4).  A sweep then waits on the latency of two
+// attempts, most of it in their random numbers and trial spins, which do not
+// depend on the lattice: both colours' are drawn together, before the first
+// update, and neighbours are decoded once per path.
+// FP64 L = 4, 256 paths: 1.31 -> 0.93 us per sweep; FP32 with 2000 paths 9.9e10 -> 1.3e11
+// attempts/s.
+template <typename Real, class Geom, bool kOne = false>
 __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, int sys_idx,
                                          int64_t path, const SweepParams& P, unsigned char* slice,
                                          int tid, int tp, int bar, Real* hbm_spins = nullptr) {
@@ -923,6 +994,50 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
 
   int accepted = 0;
   bool canceled = false;
+  if constexpr (kOne) {
+    const SpinView<Real> view[2] = {SpinView<Real>(sp, S), SpinView<Real>(sp + 3 * S, S)};
+    bool act[2];
+    int h[2], nb[2][Geom::NNB], nn[2];
+    uint32_t site[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      act[c] = tid < geo.count(c);
+      h[c] = act[c] ? tid : 0;
+      site[c] = static_cast<uint32_t>(geo.site(h[c], c, nb[c], nn[c]));
+    }
+    auto field = [&](auto c_c) {
+      constexpr int c = decltype(c_c)::value;
+      V3<Real> f{};
+#pragma unroll
+      for (int j = 0; j < Geom::NNB; ++j)
+        if (j < nn[c]) f = add3(f, view[1 - c].ld(nb[c][j]));
+      return f;
+    };
+    constexpr std::integral_constant<int, 0> c_0{};
+    constexpr std::integral_constant<int, 1> c_1{};
+    for (int64_t s = P.s_begin; s < P.s_end; ++s) {
+      const PhiloxPrefix pre = philox_prefix(static_cast<uint32_t>(s), c2, c3u, P.key);
+      const Ahead<Real> d0(philox4x32_10(site[0], pre, P.key)), d1(philox4x32_10(site[1], pre, P.key));
+      Partials<Real> part;
+      poll_cancel(P, s, tid, &cancel_flag[gidx]);
+      const bool meas = s >= P.n_therm;
+      if (meas) d0.template apply<true, false>(view[0], h[0], field(c_0), cp, act[0], accepted, part);
+      else d0.template apply<false, false>(view[0], h[0], field(c_0), cp, act[0], accepted, part);
+      group_sync(tp, bar);
+      if (cancel_flag[gidx]) {
+        canceled = true;
+        break;
+      }
+      if (meas) {
+        meter.maybe_flush(s - P.n_therm);
+        d1.template apply<true, true>(view[1], h[1], field(c_1), cp, act[1], accepted, part);
+        meter.record(part);
+      } else {
+        d1.template apply<false, false>(view[1], h[1], field(c_1), cp, act[1], accepted, part);
+      }
+      group_sync(tp, bar);
+    }
+  } else
   for (int64_t s = P.s_begin; s < P.s_end; ++s) {
     const uint32_t sw = static_cast<uint32_t>(s);
     const PhiloxPrefix pre = philox_prefix(sw, c2, c3u, P.key);
@@ -1701,6 +1816,7 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
 // switches on each work item's lattice (a batch of uneven sizes).
 constexpr int kMixedKernel = 0;
 constexpr int kChainKernel = -1;
+constexpr int kChainOneKernel = -6;  // chains with a thread for every site of a colour
 constexpr int kStreamKernel = -2;  // simple cubic lattices streamed from HBM (any even L)
 // simple cubic lattices of one size L streamed from HBM, compiled for that L
 __host__ __device__ constexpr int stream_variant(int L) { return -1000 - L; }
@@ -1715,13 +1831,22 @@ __device__ __forceinline__ void dispatch_path(const DevSystem& sy, int sys_idx, 
 // thread, which the FP64 form needs and which buys the FP32 column walk its
 // unrolled instruction-level parallelism.  (1024-thread CTAs at 64 registers
 // were measured 6-16% slower for L = 18 and 24.)
+// Two CTAs per SM (64 registers) where a lane has one site per half-sweep and
+// little to interleave: FP32 L <= 4 (one-site form, L = 4 with 40000 paths 1.27e11
+// -> 1.8e11 attempts/s; FP64 chains too take that form) and FP32 chains (64 spins,
+// 90112 paths 1.31e11 -> 1.67e11; there the one-site form gave 1.44e11, and chains
+// with more sites per lane lose 10% to the shorter register file).
+template <typename Real, int kLattice>
+constexpr bool kOneSite = kLattice == 2 || kLattice == 4 || (sizeof(Real) == 8 && kLattice == kChainOneKernel);
 template <typename Real, int kLattice>
 struct CtaLimit {
   static constexpr int value = 512;
+  static constexpr int per_sm =
+      sizeof(Real) == 4 && (kLattice == 2 || kLattice == 4 || kLattice == kChainOneKernel) ? 2 : 1;
 };
 
 template <typename Real, int kLattice>
-__global__ void __launch_bounds__(CtaLimit<Real, kLattice>::value, 1)
+__global__ void __launch_bounds__(CtaLimit<Real, kLattice>::value, CtaLimit<Real, kLattice>::per_sm)
     sweep_kernel(const SweepParams P) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int s_item;

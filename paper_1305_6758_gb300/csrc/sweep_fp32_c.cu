@@ -13,6 +13,7 @@ const void* SUFFIX(sweep_part_c)(int variant) {
     MPK_PART_CASE(24)
     MPK_PART_CASE(26)
     MPK_PART_CASE(kChainKernel)
+    MPK_PART_CASE(kChainOneKernel)
     MPK_PART_CASE(kStreamKernel)
     MPK_PART_CASE(kGlobalKernel)
     MPK_PART_CASE(stream_variant(32))

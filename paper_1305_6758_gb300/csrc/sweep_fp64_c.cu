@@ -10,6 +10,7 @@ namespace mpk {
 const void* SUFFIX(sweep_part_c)(int variant) {
   switch (variant) {
     MPK_PART_CASE(kChainKernel)
+    MPK_PART_CASE(kChainOneKernel)
     MPK_PART_CASE(kStreamKernel)
     MPK_PART_CASE(kGlobalKernel)
     MPK_PART_CASE(stream_variant(32))
