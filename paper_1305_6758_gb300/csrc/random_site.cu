@@ -211,10 +211,6 @@ __device__ void measure(const Store& S, int N, int L, uint32_t M, int lane, floa
       }
     }
   }
-  part.eb.add_warp();
-  part.mx.add_warp();
-  part.my.add_warp();
-  part.mz.add_warp();
 }
 
 template <typename Real, bool kShared, bool kChain>
@@ -279,8 +275,8 @@ __device__ void run_path_random(const DevSystem* sy, int sys_idx, int64_t path, 
     // e, m_x, m_y, m_z per site: lanes 0 to 3 divide one each
     double v;
     if constexpr (sizeof(Real) == 8) {
-      const Wide w = lane == 0 ? part.eb : lane == 1 ? part.mx : lane == 2 ? part.my : part.mz;
-      v = w.real() * (lane == 0 ? kEnergyUnit : kSpinUnit);
+      // lanes 0 .. 3: bonds, M_x, M_y, M_z
+      v = warp_sums(part.eb, part.my, part.mx, part.mz, lane).real(lane == 0 ? kEnergyBits : kFixBits);
       const double Mz = __shfl_sync(0xffffffffu, v, 3);
       if (lane == 0) v = __dsub_rn(__dmul_rn(-sy->J, v), __dmul_rn(sy->h, Mz));
     } else {

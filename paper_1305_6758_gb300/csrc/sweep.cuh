@@ -273,6 +273,12 @@ struct Wide {
       add(a, b, c);
     }
   }
+  // The value in units of 2^-unit as a double (the scale goes into the exponent).
+  __device__ __forceinline__ double real(int unit) const {
+    const double d = real();
+    const int hi = __double2hiint(d);
+    return hi == 0 ? 0.0 : __hiloint2double(hi - (unit << 20), __double2loint(d));
+  }
   // The value as a double.
   __device__ __forceinline__ double real() const {
     const int64_t low = static_cast<int64_t>((static_cast<uint64_t>(w1) << 32) | w0);
@@ -282,6 +288,40 @@ struct Wide {
     return d;
   }
 };
+
+// Sums of four values over the warp: lane l gets that of value (l & 3), in the
+// order a, c, b, d.  Two exchanges halve what a lane carries, so 18 words are
+// shuffled instead of the 60 of four butterflies.
+__device__ __forceinline__ Wide warp_sums(const Wide& a, const Wide& b, const Wide& c, const Wide& d, int lane) {
+  auto pick = [](bool second, const Wide& x, const Wide& y) {
+    Wide r;
+    r.w0 = second ? y.w0 : x.w0;
+    r.w1 = second ? y.w1 : x.w1;
+    r.w2 = second ? y.w2 : x.w2;
+    return r;
+  };
+  auto from = [](const Wide& x, int o) {
+    Wide r;
+    r.w0 = __shfl_xor_sync(0xffffffffu, x.w0, o);
+    r.w1 = __shfl_xor_sync(0xffffffffu, x.w1, o);
+    r.w2 = __shfl_xor_sync(0xffffffffu, x.w2, o);
+    return r;
+  };
+  const bool odd = lane & 1, high = lane & 2;
+  Wide x = pick(odd, a, c), y = pick(odd, b, d);  // even lanes a, b; odd lanes c, d
+  const Wide xs = from(pick(odd, c, a), 1), ys = from(pick(odd, d, b), 1);
+  x.add(xs.w0, xs.w1, xs.w2);
+  y.add(ys.w0, ys.w1, ys.w2);
+  Wide z = pick(high, x, y);
+  const Wide zs = from(pick(high, y, x), 2);
+  z.add(zs.w0, zs.w1, zs.w2);
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) {
+    const Wide t = from(z, o);
+    z.add(t.w0, t.w1, t.w2);
+  }
+  return z;
+}
 
 // Per-thread partial sums of the measurement of one sweep: sums of S . h over
 // the colour-1 sites and of the new spins.  FP64 form: exact integers, the
@@ -294,6 +334,7 @@ template <>
 struct Partials<double> {
   Wide eb, mx, my, mz;
 };
+constexpr int kEnergyBits = 57;
 constexpr double kEnergyUnit = 0x1p-57, kSpinUnit = 0x1p-53;
 
 // ------------------------------------------------------------ spin views --
@@ -760,12 +801,11 @@ struct Meter {
   // the next (every lane calls, once per measurement sweep, in order).
   // FP64 form: the warp's sums are exact integers; lane k < 4 rounds sum k.
   __device__ void record(Partials<double> part) {
-    part.eb.add_warp();
-    part.mx.add_warp();
-    part.my.add_warp();
-    part.mz.add_warp();
-    const double d = (lane == 0 ? part.eb : lane == 1 ? part.mx : lane == 2 ? part.my : part.mz).real();
-    if (lane < 4) (cur_slot() + (slot_off + warp) * kRedSlots)[lane] = d * (lane == 0 ? kEnergyUnit : kSpinUnit);
+    // lanes 0 .. 3: E, M_y, M_x, M_z
+    const Wide v = warp_sums(part.eb, part.mx, part.my, part.mz, lane);
+    if (lane < 4)
+      (cur_slot() + (slot_off + warp) * kRedSlots)[lane == 1 ? 2 : lane == 2 ? 1 : lane] =
+          v.real(lane == 0 ? kEnergyBits : kFixBits);
     advance();
   }
   __device__ void record(Partials<float> part) {
@@ -786,11 +826,53 @@ struct Meter {
     }
     advance();
   }
+  // The same by one warp in a third of the FP64 instructions (76 cycles each,
+  // and a small lattice's flush is a good part of its sweeps): lanes l and
+  // l + 16 take sweep j0 + l, each half of the observables, and the 16 sweeps
+  // are summed by exchanges that halve what a lane carries.
+  __device__ void flush_warp(int64_t j0, int n) const {
+    Real e = Real(0), ex = Real(0), ey = Real(0), ez = Real(0);
+    const int l = lane & 15;
+    const bool upper = lane >= 16;
+    if (l < n) observe(slot(j0 + l), e, ex, ey, ez);
+    const Real m2 = Arith<Real>::square(ex, ey, ez), m = sqrt(m2);
+    // lower half: E E2 M M2 M4 MX MY; upper half: MZ MZ2 |MZ| EM EMZ MMZ
+    Real v[8];
+    const Real p = upper ? ez : e;
+    v[0] = p;
+    v[1] = p * p;
+    v[2] = upper ? fabs(ez) : m;
+    v[3] = upper ? e * m : m2;
+    v[4] = upper ? e * ez : m2 * m2;
+    v[5] = upper ? m * ez : ex;
+    v[6] = upper ? Real(0) : ey;
+    v[7] = Real(0);
+#pragma unroll
+    for (int w = 4; w >= 1; w >>= 1) {  // lane bit w: keep the upper w values, give away the lower
+      const bool up = lane & w;
+#pragma unroll
+      for (int k = 0; k < w; ++k) {
+        const Real give = up ? v[k] : v[k + w], keep = up ? v[k + w] : v[k];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+      }
+    }
+    const Real total = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 8);  // value (lane & 7) of this half
+    const int at = (lane & 7) + (upper ? static_cast<int>(MP_R_MZ) : static_cast<int>(MP_R_E));
+    static_assert(MP_R_MY == 6 && MP_R_MZ == 7 && MP_R_MMZ == 12, "record order");
+    if (!(lane & 8) && (lane & 7) < (upper ? 6 : 7)) acc[at] += total;
+  }
   // Flush sweeps j0 .. j0+n-1 (one ring half): lane l takes sweep j0+l; warp
   // w owns observables w, w + warps, ...; each owned observable is summed
   // over the lanes and added to its FP64 accumulator.
+  // FP64 form with one warp and a ring of 16: flush_warp.
   __device__ void flush(int64_t j0, int n) const {
     using A = Arith<Real>;
+    if constexpr (sizeof(Real) == 8) {
+      if (nwarps == 1 && nslot == 1 && R == 16) {
+        flush_warp(j0, n);
+        return;
+      }
+    }
     Real e = Real(0), ex = Real(0), ey = Real(0), ez = Real(0);
     if (lane < n) observe(slot(j0 + lane), e, ex, ey, ez);
     Real m2;
