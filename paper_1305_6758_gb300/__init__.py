@@ -249,12 +249,14 @@ class Simulation:
         cfg.threads_per_path = threads_per_path
         self.n_therm, self.n_meas, self.precision = n_therm, n_meas, precision
         self._h = ctypes.c_void_p()
+        self._records = None  # view of the handle's record buffer (its address is fixed)
         with torch.cuda.device(self.device):
             _check(lib.mp_create_ex(ctypes.byref(cfg), ctypes.byref(self._h)))
 
     # -- lifecycle
     def close(self):
         if getattr(self, "_h", None) and self._h.value:
+            self._records = None
             _lib.mp_destroy(self._h)
             self._h = ctypes.c_void_p()
 
@@ -285,9 +287,9 @@ class Simulation:
         _check(_lib.mp_set_seed(self._h, seed), self._h)
 
     def estimates(self, system: int = 0) -> dict:
-        out = MPEstimates()
-        _check(_lib.mp_estimates(self._h, system, ctypes.byref(out)), self._h)
-        return {f: getattr(out, f) for f in EST_FIELDS}
+        out = (ctypes.c_double * NEST)()  # an mp_estimates_t: doubles only
+        _check(_lib.mp_estimates(self._h, system, ctypes.cast(out, ctypes.POINTER(MPEstimates))), self._h)
+        return dict(zip(EST_FIELDS, out))
 
     def paths(self, system: int = 0) -> np.ndarray:
         """Per-path records of one system, shape (n_paths, NREC)."""
@@ -307,10 +309,12 @@ class Simulation:
 
     def device_records(self):
         """The handle's per-path records as a (total_paths, NREC) float64 CUDA tensor view."""
-        rec = ctypes.c_void_p()
-        _check(_lib.mp_device_buffers(self._h, ctypes.byref(rec), None), self._h)
-        total = sum(s.n_paths for s in self.systems)
-        return _wrap_device(rec.value, (total, NREC), self.device)
+        if self._records is None:
+            rec = ctypes.c_void_p()
+            _check(_lib.mp_device_buffers(self._h, ctypes.byref(rec), None), self._h)
+            total = sum(s.n_paths for s in self.systems)
+            self._records = _wrap_device(rec.value, (total, NREC), self.device)
+        return self._records
 
     def backward(self, g_e, g_m):
         """Fluctuation-formula gradients (d/dbeta, d/dh) of g_e.<e> + g_m.<|m|> per system."""

@@ -16,6 +16,8 @@
 #include <mutex>
 #include <string>
 #include <tuple>
+#include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "kernels.h"
@@ -160,6 +162,8 @@ struct mp_state {
   int variant = 0;  // sweep kernel variant (see kernels.h)
   RandomSitePlan random;  // launch shape of the random-site order
 
+  unsigned char* d_tables = nullptr;  // the plan's tables (upload_tables places them)
+  size_t tables_capacity = 0;
   DevSystem* d_sys = nullptr;
   WorkItem* d_items = nullptr;
   int* d_queue = nullptr;
@@ -186,12 +190,20 @@ struct mp_state {
   int64_t sweeps_done = 0;         // progress of the resumable schedule
   int* h_cancel = nullptr;         // host-mapped cancel flag
   int* d_cancel = nullptr;
+  int cancel_slot = -1;            // its slot in the process's pool, -1: an allocation of its own
   int64_t lattice_stride = 0;      // bytes per (CTA, group) lattice buffer
   int lattice_groups = 0;          // buffers per CTA
   std::vector<void*> owned;
 
   cudaGraphExec_t gexec = nullptr;
   bool graph_dirty = true;
+  bool launched = false;           // mp_run has run with the current seed (a graph is made from the second run on)
+  // estimates and error word of the last run, read together (mp_estimates)
+  std::vector<double> est_host;
+  uint64_t runs = 0, est_run = 0;  // runs queued; the run est_host holds
+  double est_elapsed = 0.0;
+  int est_error = 0;
+  bool est_exposed = false;        // the caller has the estimates' device pointer
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
   bool ran = false;
   std::string err;
@@ -257,6 +269,51 @@ void dev_free(mp_state* h, void* p) {
   else cudaFree(p);
 }
 
+// The handles' cancel flags: host memory the kernels can read while they run.
+// Pinned allocations cost 0.1 ms each way, so flags come from one block of
+// kCancelSlots cache lines per process, and return to it; handles beyond that
+// allocate their own.
+constexpr int kCancelSlots = 256, kCancelStride = 64 / static_cast<int>(sizeof(int));
+std::mutex g_cancel_mu;
+int* g_cancel_base = nullptr;
+std::vector<int> g_cancel_free;
+
+cudaError_t cancel_acquire(mp_state* h) {
+  {
+    std::lock_guard<std::mutex> lock(g_cancel_mu);
+    if (!g_cancel_base) {
+      void* p = nullptr;
+      const cudaError_t e = cudaHostAlloc(&p, kCancelSlots * kCancelStride * sizeof(int),
+                                          cudaHostAllocMapped | cudaHostAllocPortable);
+      if (e != cudaSuccess) return e;
+      g_cancel_base = static_cast<int*>(p);
+      for (int k = kCancelSlots - 1; k >= 0; --k) g_cancel_free.push_back(k);
+    }
+    if (!g_cancel_free.empty()) {
+      h->cancel_slot = g_cancel_free.back();
+      g_cancel_free.pop_back();
+      h->h_cancel = g_cancel_base + h->cancel_slot * kCancelStride;
+    }
+  }
+  if (h->cancel_slot < 0) {
+    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&h->h_cancel), sizeof(int), cudaHostAllocMapped);
+    if (e != cudaSuccess) return e;
+  }
+  *h->h_cancel = 0;
+  return cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->d_cancel), h->h_cancel, 0);
+}
+
+void cancel_release(mp_state* h) {  // after the handle's stream has drained
+  if (!h->h_cancel) return;
+  if (h->cancel_slot < 0) {
+    cudaFreeHost(h->h_cancel);
+  } else {
+    std::lock_guard<std::mutex> lock(g_cancel_mu);
+    g_cancel_free.push_back(h->cancel_slot);
+  }
+  h->h_cancel = nullptr;
+}
+
 void release(mp_state* h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
@@ -267,7 +324,7 @@ void release(mp_state* h) {
     else cudaFree(p);
   }
   h->owned.clear();
-  if (h->h_cancel) cudaFreeHost(h->h_cancel);
+  cancel_release(h);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
@@ -775,23 +832,28 @@ int upload_tables(mp_state* h, const std::vector<WorkItem>& items, bool with_pai
     d.unit_K = K;
     d.unit_U = U;
   }
-  int64_t bytes = 0;
-  auto copy = [&](void* dst, const void* src, size_t b) {
-    bytes += static_cast<int64_t>(b);
-    return cudaMemcpyAsync(dst, src, b, cudaMemcpyHostToDevice, h->stream);
+  // the tables one after another in their region, in one copy
+  std::vector<unsigned char> stage;
+  auto put = [&](auto** dst, const void* src, size_t b) {
+    const size_t at = stage.size();
+    *dst = reinterpret_cast<std::remove_pointer_t<decltype(dst)>>(h->d_tables + at);
+    stage.resize(at + (b + 255) / 256 * 256);
+    if (b) std::memcpy(stage.data() + at, src, b);
   };
-  MP_CUDA(h, copy(h->d_sys, h->hsys.data(), sizeof(DevSystem) * n));
-  if (!items.empty()) MP_CUDA(h, copy(h->d_items, items.data(), sizeof(WorkItem) * items.size()));
-  if (with_pairs && !h->pair_items.empty())
-    MP_CUDA(h, copy(h->d_items + items.size(), h->pair_items.data(), sizeof(WorkItem) * h->pair_items.size()));
-  MP_CUDA(h, copy(h->d_spin_offset, h->spin_offset.data(), sizeof(int64_t) * n));
   std::vector<unsigned long long> thr(10 * static_cast<size_t>(n), 0ull);
   for (int k = 0; k < n; ++k)
     if (h->systems[k].lattice == MP_LATTICE_ISING) ising_thresholds(h->systems[k], &thr[10 * k]);
-  MP_CUDA(h, copy(h->d_thr, thr.data(), sizeof(unsigned long long) * thr.size()));
-  if (!units.empty()) MP_CUDA(h, copy(h->d_units, units.data(), sizeof(int4) * units.size()));
+  std::vector<WorkItem> all(items);
+  if (with_pairs) all.insert(all.end(), h->pair_items.begin(), h->pair_items.end());
+  put(&h->d_sys, h->hsys.data(), sizeof(DevSystem) * n);
+  put(&h->d_spin_offset, h->spin_offset.data(), sizeof(int64_t) * n);
+  put(&h->d_thr, thr.data(), sizeof(unsigned long long) * thr.size());
+  put(&h->d_units, units.data(), sizeof(int4) * units.size());
+  put(&h->d_items, all.data(), sizeof(WorkItem) * all.size());
+  if (stage.size() > h->tables_capacity) return fail(h, MP_ENOMEM, "no room for the plan's tables");
+  MP_CUDA(h, cudaMemcpyAsync(h->d_tables, stage.data(), stage.size(), cudaMemcpyHostToDevice, h->stream));
   MP_CUDA(h, cudaStreamSynchronize(h->stream));
-  h->upload_bytes = bytes;
+  h->upload_bytes = static_cast<int64_t>(stage.size());
   return MP_OK;
 }
 
@@ -958,14 +1020,19 @@ int autotune(mp_state* h, const mp_config* cfg) {
   return rc;
 }
 
-// After the stream has drained: MP_ETIMEOUT if a kernel's bounded wait gave up.
-int check_error_flag(mp_state* h) {
-  int flag = 0;
-  MP_CUDA(h, cudaMemcpy(&flag, h->d_error, sizeof(int), cudaMemcpyDeviceToHost));
+// The status of a run's error word: MP_ETIMEOUT if a kernel's bounded wait gave up.
+int error_status(mp_state* h, int flag) {
   if (flag == kErrCanceled) return fail(h, MP_ECANCELED, "the run was canceled; results invalid");
   if (flag == kErrLaunch) return fail(h, MP_ECUDA, "two-CTA cluster paths ran without a cluster launch");
   if (flag) return fail(h, MP_ETIMEOUT, "a bulk copy did not complete in time; results invalid");
   return MP_OK;
+}
+
+// After the stream has drained.
+int check_error_flag(mp_state* h) {
+  int flag = 0;
+  MP_CUDA(h, cudaMemcpy(&flag, h->d_error, sizeof(int), cudaMemcpyDeviceToHost));
+  return error_status(h, flag);
 }
 
 extern "C" {
@@ -1026,32 +1093,36 @@ int mp_create_ex(const mp_config* cfg, mp_handle* out) {
     cudaError_t ce = cudaEventCreate(&e);
     if (ce != cudaSuccess) return bail(cuda_fail(h, ce, "cudaEventCreate"));
   }
-  {  // the cancel flag: host memory the kernels can read while they run
-    cudaError_t ce = cudaHostAlloc(reinterpret_cast<void**>(&h->h_cancel), sizeof(int), cudaHostAllocMapped);
-    if (ce != cudaSuccess) return bail(cuda_fail(h, ce, "cudaHostAlloc"));
-    *h->h_cancel = 0;
-    ce = cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->d_cancel), h->h_cancel, 0);
-    if (ce != cudaSuccess) return bail(cuda_fail(h, ce, "cudaHostGetDevicePointer"));
+  {
+    const cudaError_t ce = cancel_acquire(h);
+    if (ce != cudaSuccess) return bail(cuda_fail(h, ce, "cancel flag"));
   }
   const int n = static_cast<int>(h->hsys.size());
-  h->d_sys = static_cast<DevSystem*>(dev_alloc(h, sizeof(DevSystem) * n));
-  h->d_items = static_cast<WorkItem*>(dev_alloc(h, sizeof(WorkItem) * h->total_paths));  // any plan fits
-  h->d_queue = static_cast<int*>(dev_alloc(h, 256));
-  h->d_rec = static_cast<double*>(dev_alloc(h, sizeof(double) * MP_NREC * h->total_paths));
-  h->d_est = static_cast<double*>(dev_alloc(h, sizeof(double) * MP_NEST * n));
-  h->d_work = static_cast<double*>(dev_alloc(h, sizeof(double) * reduce_work_doubles(h->total_paths, n)));
-  h->d_spin_offset = static_cast<int64_t*>(dev_alloc(h, sizeof(int64_t) * n));
-  h->d_thr = static_cast<unsigned long long*>(dev_alloc(h, sizeof(unsigned long long) * 10 * n));
   // unit tables: at most L^3/2 units per simple cubic size that fits shared memory
   h->units_capacity = 0;
   for (const mp_system& s : h->systems)
     if (s.lattice == MP_LATTICE_SC && s.L <= 26) h->units_capacity += static_cast<int64_t>(s.L) * s.L * s.L / 2;
-  h->d_units = h->units_capacity > 0 ? static_cast<int4*>(dev_alloc(h, sizeof(int4) * h->units_capacity)) : nullptr;
-  if (!h->d_sys || !h->d_items || !h->d_queue || !h->d_rec || !h->d_est || !h->d_work ||
-      !h->d_spin_offset || !h->d_thr || (h->units_capacity > 0 && !h->d_units))
-    return bail(fail(h, MP_ENOMEM, "device allocation failed"));
-  h->d_error = static_cast<int*>(dev_alloc(h, 256));
-  if (!h->d_error) return bail(fail(h, MP_ENOMEM, "device allocation failed"));
+  {  // one allocation: the tables (uploaded together), the queue, records, scratch, estimates and error word
+    size_t size = 0;
+    std::vector<std::pair<void**, size_t>> parts;
+    auto part = [&](auto** p, size_t bytes) {
+      parts.emplace_back(reinterpret_cast<void**>(p), size);
+      size += (bytes + 255) / 256 * 256;
+    };
+    const size_t paths = static_cast<size_t>(h->total_paths), ns = static_cast<size_t>(n);
+    // (a work item per path at most: any plan fits)
+    h->tables_capacity = (sizeof(DevSystem) + sizeof(int64_t) + sizeof(unsigned long long) * 10) * ns +
+                         sizeof(int4) * static_cast<size_t>(h->units_capacity) + sizeof(WorkItem) * paths + 5 * 256;
+    part(&h->d_tables, h->tables_capacity);
+    part(&h->d_queue, 256);
+    part(&h->d_rec, sizeof(double) * MP_NREC * paths);
+    part(&h->d_work, sizeof(double) * static_cast<size_t>(reduce_work_doubles(h->total_paths, n)));
+    part(&h->d_est, sizeof(double) * MP_NEST * ns);
+    part(&h->d_error, 256);
+    unsigned char* base = static_cast<unsigned char*>(dev_alloc(h, size));
+    if (!base) return bail(fail(h, MP_ENOMEM, "device allocation failed"));
+    for (auto& p : parts) *p.first = base + p.second;
+  }
   if (h->max_paths > MP_R_MAX_PATHS) {  // sorting space for r beyond shared memory
     h->d_sort = static_cast<double*>(dev_alloc(h, sizeof(double) * 2 * h->total_paths));
     if (!h->d_sort) return bail(fail(h, MP_ENOMEM, "sort buffer allocation failed"));
@@ -1075,7 +1146,18 @@ int mp_create_ex(const mp_config* cfg, mp_handle* out) {
 int mp_run(mp_handle h) {
   if (!h) return fail(nullptr, MP_EINVAL, "handle is NULL");
   DeviceGuard dg(h->device);
-  if (!(h->flags & MP_FLAG_GRAPH)) {
+  // A graph pays from the second run with the same seed on: the first one is
+  // launched directly (unless the caller is capturing the stream, which a
+  // handle with MP_FLAG_GRAPH refuses, below).
+  bool direct = !(h->flags & MP_FLAG_GRAPH);
+  if (!direct && !h->launched) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    MP_CUDA(h, cudaStreamIsCapturing(h->stream, &cs));
+    direct = cs == cudaStreamCaptureStatusNone;
+    h->launched = direct;
+  }
+  ++h->runs;
+  if (direct) {
     *h->h_cancel = 0;
     int rc = enqueue_run(h, 0, h->n_therm + h->n_meas, false, false);
     if (rc != MP_OK) return rc;
@@ -1112,6 +1194,7 @@ int mp_set_seed(mp_handle h, uint64_t seed) {
   if (seed != h->seed) {
     h->seed = seed;
     h->graph_dirty = true;
+    h->launched = false;
   }
   return MP_OK;
 }
@@ -1122,13 +1205,33 @@ int mp_estimates(mp_handle h, int system, mp_estimates_t* out) {
     return fail(h, MP_EINVAL, "bad system index %d or NULL output", system);
   if (!h->ran) return fail(h, MP_ESTATE, "no run yet");
   DeviceGuard dg(h->device);
-  MP_CUDA(h, cudaMemcpyAsync(out, h->d_est + static_cast<int64_t>(system) * MP_NEST,
-                             sizeof(mp_estimates_t), cudaMemcpyDeviceToHost, h->stream));
-  MP_CUDA(h, cudaStreamSynchronize(h->stream));
-  float ms = 0.f;  // sweep and reduction kernels of the last run
-  out->elapsed_s = cudaEventElapsedTime(&ms, h->ev[0], h->ev[2]) == cudaSuccess ? 1e-3 * ms : NAN;
-  cudaGetLastError();
-  return check_error_flag(h);
+  // Every system's estimates of a run and its error word come in one copy
+  // (they lie side by side), 29 us saved for each system after the first.  Not
+  // once the caller has their device pointer and may write through it.
+  const size_t n = h->hsys.size(), count = n * MP_NEST + 1;
+  if (n > 1024 || h->est_exposed) {
+    MP_CUDA(h, cudaMemcpyAsync(out, h->d_est + static_cast<int64_t>(system) * MP_NEST,
+                               sizeof(mp_estimates_t), cudaMemcpyDeviceToHost, h->stream));
+    MP_CUDA(h, cudaStreamSynchronize(h->stream));
+    float ms = 0.f;  // sweep and reduction kernels of the last run
+    out->elapsed_s = cudaEventElapsedTime(&ms, h->ev[0], h->ev[2]) == cudaSuccess ? 1e-3 * ms : NAN;
+    cudaGetLastError();
+    return check_error_flag(h);
+  }
+  if (h->est_run != h->runs) {
+    h->est_host.resize(count);
+    h->est_run = 0;
+    MP_CUDA(h, cudaMemcpyAsync(h->est_host.data(), h->d_est, sizeof(double) * count, cudaMemcpyDeviceToHost, h->stream));
+    MP_CUDA(h, cudaStreamSynchronize(h->stream));
+    float ms = 0.f;
+    h->est_elapsed = cudaEventElapsedTime(&ms, h->ev[0], h->ev[2]) == cudaSuccess ? 1e-3 * ms : NAN;
+    cudaGetLastError();
+    std::memcpy(&h->est_error, &h->est_host[n * MP_NEST], sizeof(int));
+    h->est_run = h->runs;
+  }
+  std::memcpy(out, &h->est_host[static_cast<size_t>(system) * MP_NEST], sizeof(mp_estimates_t));
+  out->elapsed_s = h->est_elapsed;
+  return error_status(h, h->est_error);
 }
 
 int mp_paths(mp_handle h, int system, double* host_out, int64_t cap) {
@@ -1149,7 +1252,10 @@ int mp_paths(mp_handle h, int system, double* host_out, int64_t cap) {
 int mp_device_buffers(mp_handle h, double** d_records, double** d_estimates) {
   if (!h) return fail(nullptr, MP_EINVAL, "handle is NULL");
   if (d_records) *d_records = h->d_rec;
-  if (d_estimates) *d_estimates = h->d_est;
+  if (d_estimates) {
+    *d_estimates = h->d_est;
+    h->est_exposed = true;
+  }
   return MP_OK;
 }
 
@@ -1300,6 +1406,7 @@ int mp_run_sweeps(mp_handle h, int64_t n_sweeps) {
   if (rc != MP_OK) return rc;
   const int64_t s_end = std::min(total, h->sweeps_done + n_sweeps);
   *h->h_cancel = 0;
+  ++h->runs;
   rc = enqueue_run(h, h->sweeps_done, s_end, h->sweeps_done > 0, true);
   if (rc != MP_OK) return rc;
   MP_CUDA(h, cudaStreamSynchronize(h->stream));
