@@ -670,7 +670,65 @@ __device__ __forceinline__ void half_sweep(const Geom& geo, int c, const PhiloxP
       const int seg = LL / K;  // planes per segment
       constexpr int U = kColumnChunk<Real, Geom>;
       constexpr int NH = HP * LL;
-      for (int u = tid; u < HP * K; u += tp) {
+      // Where chunks of two give a warp too few independent random-number
+      // chains, the rounds of a thermalisation sweep are taken two at a time (u
+      // and u + tp side by side; measurement sweeps keep the order of their FP32
+      // sums, and FP64 has no registers for it: 7.3e10 -> 4.7e10 attempts/s at
+      // L = 16).  Attempts/s before -> after, sweeps of all kinds: L = 10, 1000
+      // paths (7 warps per SM) 1.36e11 -> 1.47e11, a full GPU 2.08e11 ->
+      // 2.15e11, L = 22 1.71e11 -> 1.72e11, L = 26 1.73e11 -> 1.85e11.  Chunks
+      // of three lose by it (L = 6: 1.21e11 -> 1.18e11), four rounds at a time
+      // lose everywhere.
+      int u_first = tid;
+      if constexpr (sizeof(Real) == 4 && !kMeas && U == 2 && !Geom::kInMixed) {
+        const int n_units = HP * K, rounds = (n_units + tp - 1) / tp;
+        struct Unit {
+          int hh, oyp, oym, pa, oxa, oxb;
+          bool act;
+          V3<Real> o0, mz;
+        };
+        for (; u_first < rounds / 2 * 2 * tp; u_first += 2 * tp) {
+          Unit unit[2];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            Unit& w = unit[j];
+            // the last round may lack a unit for this thread: it goes along
+            // with its other one and changes nothing
+            w.act = j == 0 || u_first + tp < n_units;
+            const int u = u_first + (j == 1 && w.act ? tp : 0);
+            const int4 d = units != nullptr ? __ldg(units + u) : column_unit(LL, K, u);
+            w.hh = d.x & 0x7fffffff;
+            w.pa = static_cast<int>(static_cast<unsigned>(d.x) >> 31) ^ c;
+            const int xa = (d.y << 8) >> 24, xb = d.y >> 24;  // signed bytes 2 and 3
+            w.oxa = c ? xb : xa;
+            w.oxb = c ? xa : xb;
+            w.oyp = d.z;
+            w.oym = d.w;
+            w.o0 = oth.ld(w.hh);
+            w.mz = oth.ld(d.y & 0xffff);
+          }
+          for (int zc = 0; zc < seg; zc += U) {
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+#pragma unroll
+              for (int j = 0; j < 2; ++j) {
+                Unit& w = unit[j];
+                const int nxo = w.hh + ((k & 1) ? w.oxb : w.oxa);
+                const int zn = (k == U - 1 && w.hh + HP >= NH) ? w.hh + HP - NH : w.hh + HP;
+                const V3<Real> cz = oth.ld(zn);
+                const V3<Real> f = add3(
+                    add3(add3(add3(add3(w.o0, oth.ld(nxo)), oth.ld(w.hh + w.oyp)), oth.ld(w.hh + w.oym)), cz), w.mz);
+                update_spin<false, false>(static_cast<uint32_t>(2 * w.hh + ((k & 1) ? w.pa ^ 1 : w.pa)), pre, key, own,
+                                          w.hh, own.ld(w.hh), f, cp, w.act, accepted, part);
+                w.mz = w.o0;
+                w.o0 = cz;
+                w.hh += HP;
+              }
+            }
+          }
+        }
+      }
+      for (int u = u_first; u < HP * K; u += tp) {
         // the unit: half index hh of its first site and of that site's -z
         // neighbour, +-y offsets, and the x parity p of the site: it flips
         // from plane to plane, so sites an even number of planes after the
