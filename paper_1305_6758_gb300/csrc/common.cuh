@@ -45,7 +45,11 @@ struct DevSystem {
   int32_t unit_K;       // column segments per column of the unit table (below)
   int64_t path_begin;   // path id (random-number counter) of the system's path 0
   int32_t unit_off;     // first entry of the system's column-walk units in SweepParams::units, or -1
-  int32_t unit_U;       // column chunk the unit table was made for
+  int32_t unit_U;       // column chunk the unit tables were made for
+  int32_t tm;           // the first tm of the tp threads add up the measured sums (0: all of them)
+  int32_t sum_K;        // their unit table, as unit_K and unit_off
+  int32_t sum_off;
+  int32_t pad;
 };
 
 constexpr int kModeShared = 0;

@@ -426,6 +426,8 @@ int plan(mp_state* h, const mp_config* cfg) {
   const double target = cta_max <= 512 ? 16.0 : 8.0;
   MP_CUDA(h, reduce_prepare());
   std::vector<int> tp(n), slice(n), ring(n);
+  std::vector<int> tw(n, 0);  // threads launched per path: tp or more (wide_threads)
+  int wide_of = -1;           // the last system that wide_threads was asked for
   // The partial-sum ring (sweeps per half): the largest power of two up to 16
   // among those that fit the most paths into one CTA -- shared memory, the
   // CTA size and the named barriers permit (a shorter ring only flushes to
@@ -448,11 +450,63 @@ int plan(mp_state* h, const mp_config* cfg) {
   int max_tp = 32;
   int64_t batch_paths = 0;
   for (const mp_system& sy : h->systems) batch_paths += sy.n_paths;
+  // FP32 simple cubic paths whose tp threads (the order of their sums) leave
+  // the SMs short of warps get c > tp: the count with the least estimated time,
+  // if that is 6% below tp's.  Estimate of a half-sweep of the `fit` paths
+  // on an SM, in cycles, from the measured rates of 1 to 16 warps at L = 6 .. 26:
+  // issue, of 150 per site and warp (175 in chunks of up to three planes) over the
+  // busiest of the four schedulers, and latency, of a thread's chunks one after
+  // another (450 each beyond their issue) and a barrier (700); whichever is
+  // longer, with some of the other.  A measurement sweep costs 7% more with tp
+  // threads, and with more the pass that makes the sums (16 per site and warp,
+  // 300 + 30 U per chunk, two colours).  Attempts/s before -> after, all
+  // sweeps but one thermalising / half of them measured, one path per SM:
+  // L = 10 2.6e10 -> 9.4e10 / 2.5e10 -> 5.1e10, L = 16 1.44e11 -> 1.96e11 /
+  // 1.30e11 -> 1.58e11, L = 20 1.15e11 -> 2.14e11 / 1.11e11 -> 1.67e11; the GPU
+  // full, L = 20 (two paths of 160 threads to an SM, now 256) 1.64e11 ->
+  // 2.12e11 / 1.60e11 -> 1.80e11, L = 12 1.73e11 -> 1.98e11 / unchanged.
+  auto wide_threads = [&](int k, int64_t lat, int NH) {
+    const int L = h->systems[k].L, U = column_chunk(4, L, variant == 0);
+    const bool pairs = U == 2 && variant != 0;  // rounds taken two at a time
+    const double site = U > 3 ? 150.0 : 175.0;
+    const double n_meas = static_cast<double>(h->n_meas), n_all = static_cast<double>(h->n_therm) + n_meas;
+    const int64_t load = (batch_paths + sms - 1) / sms;  // paths per SM
+    double best = 0.0;
+    for (int c = tp[k]; c <= std::min(cta_max, round_up(NH, 32)); c += 32) {
+      const int s = round_up(slice_spin_offset(c, ring[k]) + static_cast<int>(lat), 128);
+      int64_t fit = std::min<int64_t>(smem_max / s, c > 32 ? std::min(15, cta_max / c) : cta_max / c);
+      fit = std::min(fit, load);
+      if (fit < 1) continue;
+      const int64_t turns = (load + fit - 1) / fit;  // an SM takes its paths in turns
+      fit = (load + turns - 1) / turns;
+      const int K = column_segments(L, U, c), units = L * L / 2 * K, rounds = (units + c - 1) / c;
+      const double warps = static_cast<double>(fit) * std::min(c, round_up(units, 32)) / 32;
+      const double issue = fit * ((units + 31) / 32) * (L / K) * site / warps * std::ceil(warps / 4);
+      const double chunks = (pairs ? (rounds + 1) / 2 : rounds) * (L / K / U);
+      const double latency = chunks * ((pairs && rounds > 1 ? 2 : 1) * U * site + 450) + 700;
+      const double walk = std::cbrt(issue * issue * issue + latency * latency * latency);
+      double time = n_all * walk;
+      if (c == tp[k]) {
+        time += n_meas * 0.07 * walk;  // sums along the way
+      } else {  // the pass by tp threads that makes the sums
+        const int Km = column_segments(L, U, tp[k]), um = L * L / 2 * Km;
+        time += n_meas * 0.5 * (fit * ((um + 31) / 32) * (L / Km) * 16.0 +
+                                (um + tp[k] - 1) / tp[k] * (L / Km / U) * (300.0 + 30.0 * U) + 1000);
+      }
+      time *= (c == tp[k] ? 0.94 : 1.0) * static_cast<double>(turns);
+      if (best == 0.0 || time < best * (1.0 - 1e-9)) {
+        best = time;
+        tw[k] = c;
+        slice[k] = s;
+      }
+    }
+  };
   for (int k = 0; k < n; ++k) {
     const int64_t N = sites_of(h->systems[k]);
     const int NH = static_cast<int>((N + 1) / 2);
     int t = (static_cast<int>(h->tp_override.size()) > k && h->tp_override[k] > 0) ? h->tp_override[k]
                                                                                   : cfg->threads_per_path;
+    const bool by_default = t == 0;
     if (paired(h->systems[k], h->precision, h->flags)) {
       // one CTA of cta_max threads on each half: one column of L/2 planes per thread
       if (t != 0 && t != cta_max)
@@ -550,8 +604,18 @@ int plan(mp_state* h, const mp_config* cfg) {
     if (slice[k] > smem_max)
       return fail(h, MP_EINVAL, "system %d needs %d bytes of shared memory per path (max %d)", k,
                   slice[k], smem_max);
-    max_tp = std::max(max_tp, t);
+    if (by_default && real == 4 && h->systems[k].lattice == MP_LATTICE_SC) {
+      if (wide_of >= 0 && h->systems[wide_of].L == h->systems[k].L) {  // the same size as the one before
+        tw[k] = tw[wide_of];
+        slice[k] = slice[wide_of];
+      } else {
+        wide_threads(k, lat, NH);
+      }
+      wide_of = k;
+    }
+    max_tp = std::max(max_tp, std::max(t, tw[k]));
   }
+  for (int k = 0; k < n; ++k) tw[k] = std::max(tw[k], tp[k]);
   if (variant == -1) {  // chains with one site of a colour per thread have their own kernel
     bool one = true;
     for (int k = 0; k < n; ++k) one = one && (sites_of(h->systems[k]) + 1) / 2 <= tp[k];
@@ -563,8 +627,8 @@ int plan(mp_state* h, const mp_config* cfg) {
   }
   auto paths_per_cta = [&](int k, int cta) {
     if (paired(h->systems[k], h->precision, h->flags)) return 1;  // one path per cluster
-    int g = cta / tp[k];
-    if (tp[k] > 32) g = std::min(g, 15);  // named barriers 1..15
+    int g = cta / tw[k];
+    if (tw[k] > 32) g = std::min(g, 15);  // named barriers 1..15
     g = std::min<int64_t>(g, smem_max / slice[k]);
     g = static_cast<int>(std::min<int64_t>(g, h->systems[k].n_paths));
     return std::max(g, 1);
@@ -585,7 +649,15 @@ int plan(mp_state* h, const mp_config* cfg) {
     // Ising paths all take equally long, so the last round of a launch is
     // partly empty: small CTAs spread its paths over every SM (four to an SM,
     // each with 16 of its 64 named barriers)
-    if (variant == kIsingKernel) cta = std::max(max_tp, 256);
+    if (variant == kIsingKernel) {
+      cta = std::max(max_tp, 256);
+    } else if (cta < cta_max) {
+      // no threads beyond the paths': with 160 a path, 450 paths of L = 12,
+      // three CTAs of 160 to an SM and not two of 256
+      int used = max_tp;
+      for (int k = 0; k < n; ++k) used = std::max(used, paths_per_cta(k, cta) * tw[k]);
+      cta = std::min(cta, used);
+    }
   }
   if (cta < max_tp) return fail(h, MP_EINVAL, "cta_threads %d below threads per path %d", cta, max_tp);
 
@@ -609,7 +681,10 @@ int plan(mp_state* h, const mp_config* cfg) {
     d.L = s.L;
     d.N = static_cast<int32_t>(sites_of(s));
     d.NH = (d.N + 1) / 2;
-    d.tp = tp[k];
+    d.tp = tw[k];
+    d.tm = tw[k] > tp[k] ? tp[k] : 0;
+    d.sum_K = 0;
+    d.sum_off = -1;
     d.g = paths_per_cta(k, cta);
     d.slice_bytes = slice[k];
     d.ring = ring[k];
@@ -819,17 +894,21 @@ int upload_tables(mp_state* h, const std::vector<WorkItem>& items, bool with_pai
         d.mode != kModeShared)
       continue;
     const int U = column_chunk(real, d.L, mixed);
-    const int K = column_segments(d.L, U, d.tp);
-    const int n_units = d.L * d.L / 2 * K;
-    auto it = unit_at.find(std::make_tuple(d.L, K, U));
-    if (it == unit_at.end()) {
-      if (static_cast<int64_t>(units.size()) + n_units > h->units_capacity)
-        return fail(h, MP_ENOMEM, "system %d: no room for its column-walk unit table", k);
-      it = unit_at.emplace(std::make_tuple(d.L, K, U), static_cast<int>(units.size())).first;
-      for (int u = 0; u < n_units; ++u) units.push_back(column_unit(d.L, K, u));
+    // the table of tp threads, and that of the tm threads which add up the sums
+    for (const int t : {d.tp, d.tm}) {
+      if (t == 0) continue;
+      const int K = column_segments(d.L, U, t);
+      const int n_units = d.L * d.L / 2 * K;
+      auto it = unit_at.find(std::make_tuple(d.L, K, U));
+      if (it == unit_at.end()) {
+        if (static_cast<int64_t>(units.size()) + n_units > h->units_capacity)
+          return fail(h, MP_ENOMEM, "system %d: no room for its column-walk unit table", k);
+        it = unit_at.emplace(std::make_tuple(d.L, K, U), static_cast<int>(units.size())).first;
+        for (int u = 0; u < n_units; ++u) units.push_back(column_unit(d.L, K, u));
+      }
+      (t == d.tp ? d.unit_off : d.sum_off) = it->second;
+      (t == d.tp ? d.unit_K : d.sum_K) = K;
     }
-    d.unit_off = it->second;
-    d.unit_K = K;
     d.unit_U = U;
   }
   // the tables one after another in their region, in one copy
@@ -1101,7 +1180,7 @@ int mp_create_ex(const mp_config* cfg, mp_handle* out) {
   // unit tables: at most L^3/2 units per simple cubic size that fits shared memory
   h->units_capacity = 0;
   for (const mp_system& s : h->systems)
-    if (s.lattice == MP_LATTICE_SC && s.L <= 26) h->units_capacity += static_cast<int64_t>(s.L) * s.L * s.L / 2;
+    if (s.lattice == MP_LATTICE_SC && s.L <= 26) h->units_capacity += static_cast<int64_t>(s.L) * s.L * s.L;
   {  // one allocation: the tables (uploaded together), the queue, records, scratch, estimates and error word
     size_t size = 0;
     std::vector<std::pair<void**, size_t>> parts;
@@ -1482,7 +1561,8 @@ int mp_system_plan(mp_handle h, int system, int* threads_per_path, int* paths_pe
   if (system < 0 || system >= static_cast<int>(h->hsys.size()))
     return fail(h, MP_EINVAL, "bad system index %d", system);
   const DevSystem& d = h->hsys[system];
-  if (threads_per_path) *threads_per_path = d.tp;
+  // the count that orders a path's sums (wide_threads may launch more)
+  if (threads_per_path) *threads_per_path = d.tm > 0 ? d.tm : d.tp;
   if (paths_per_cta) *paths_per_cta = d.g;
   // 0 shared memory, 1 streamed from HBM, 2 two-CTA cluster, 3 in place in HBM
   if (streamed_from_hbm) *streamed_from_hbm = d.mode;

@@ -804,6 +804,65 @@ __device__ __forceinline__ void half_sweep(const Geom& geo, int c, const PhiloxP
   }
 }
 
+// The sums that a measurement half-sweep of tm threads adds up, from the spins
+// after the sweep, in the same order: colour 0's magnetisation, or (kBonds)
+// colour 1's and, with its local fields, the bond energy.  Bound by latency (only
+// tm threads have work): a unit's table entry is fetched one unit ahead and a
+// chunk's spins before its first addition.
+template <class Geom, bool kBonds>
+__device__ __forceinline__ void sum_sites(const Geom& geo, const float* sp, int tid, int tm, int K, const int4* units,
+                                          Partials<float>& part) {
+  constexpr int HP = Geom::HP, LL = 2 * Geom::HL, NH = HP * LL;
+  // planes taken together: a whole chunk, or a part of it (U = 8 and 6: half)
+  constexpr int kChunk = kColumnChunk<float, Geom>, U = kChunk % 4 == 0 ? 4 : kChunk % 3 == 0 ? 3 : kChunk;
+  constexpr int c = kBonds ? 1 : 0;
+  const int S = geo.stride(), seg = LL / K;
+  const SpinView<float> own(const_cast<float*>(sp) + c * 3 * S, S), oth(const_cast<float*>(sp) + (1 - c) * 3 * S, S);
+  // each unit's table entry is fetched while the one before is added up
+  auto entry = [&](int u) { return units != nullptr ? __ldg(units + u) : column_unit(LL, K, u); };
+  int4 next = tid < HP * K ? entry(tid) : int4{};
+#pragma unroll 1
+  for (int u = tid; u < HP * K; u += tm) {
+    const int4 d = next;
+    if (u + tm < HP * K) next = entry(u + tm);
+    int hh = d.x & 0x7fffffff;
+    int oxa = d.y >> 24, oxb = (d.y << 8) >> 24;  // colour 1's
+    V3<float> o0{}, mz{};
+    if constexpr (kBonds) {
+      o0 = oth.ld(hh);
+      mz = oth.ld(d.y & 0xffff);
+    }
+#pragma unroll 1
+    for (int zc = 0; zc < seg; zc += U) {
+      V3<float> n[U], f[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k, hh += HP) {
+        n[k] = own.ld(hh);
+        if constexpr (kBonds) {
+          const int nxo = hh + ((k & 1) ? oxb : oxa);
+          const int zn = (k == U - 1 && hh + HP >= NH) ? hh + HP - NH : hh + HP;
+          const V3<float> cz = oth.ld(zn);
+          f[k] = add3(add3(add3(add3(add3(o0, oth.ld(nxo)), oth.ld(hh + d.z)), oth.ld(hh + d.w)), cz), mz);
+          mz = o0;
+          o0 = cz;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        part.mx += n[k].x;
+        part.my += n[k].y;
+        part.mz += n[k].z;
+        if constexpr (kBonds) part.eb += Arith<float>::dot(n[k].x, n[k].y, n[k].z, f[k].x, f[k].y, f[k].z);
+      }
+      if constexpr (U & 1) {
+        const int t = oxa;
+        oxa = oxb;
+        oxb = t;
+      }
+    }
+  }
+}
+
 // ----------------------------------------------------------- measurement --
 // Per-path measurement state in the path's shared-memory slice: the FP64
 // accumulators and the partial-sum ring.  ring[half][slot][warp][4] holds each
@@ -987,11 +1046,12 @@ struct Meter {
       acc[MP_R_FE] = static_cast<double>(e);
     }
   }
-  // Reduce the acceptance count and the worst | |S| - 1 | over the group and
+  // Reduce the acceptance count and the worst | |S| - 1 | over the group's warps
+  // (nwarps, or all_warps of a wide path) and
   // write the path's record (the ring area is reused; call after a barrier).
   __device__ void write_record(double* rec, int accepted, double worst, int64_t nsweeps,
                                int64_t n_meas, int N, int tp, int bar, double accepted_before,
-                               double* save_accepted) const {
+                               double* save_accepted, int all_warps = 0) const {
     double nacc = static_cast<double>(accepted);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1006,7 +1066,7 @@ struct Meter {
     group_sync(tp, bar);
     if (tid == 0) {
       double tot = accepted_before, wmax = 0.0;
-      for (int w = 0; w < nwarps; ++w) {
+      for (int w = 0; w < (all_warps > 0 ? all_warps : nwarps); ++w) {
         tot += fin[2 * w + 0];
         wmax = fmax(wmax, fin[2 * w + 1]);
       }
@@ -1057,6 +1117,14 @@ __device__ __forceinline__ void poll_cancel(const SweepParams& P, int64_t s, int
   }
 }
 
+// Each thread group's cancel verdict; one array for all paths of a geometry
+// (a second one would take shared memory, and rings of partial sums, from them).
+template <typename Real, class Geom>
+__device__ __forceinline__ int* cancel_flags() {
+  __shared__ int flags[kMaxGroups];
+  return flags;
+}
+
 // ------------------------------------------------------------- one path --
 // The lattice lives in the slice's shared memory, or in HBM at `hbm_spins`
 // (the same layout) when it is updated in place there.
@@ -1068,11 +1136,23 @@ __device__ __forceinline__ void poll_cancel(const SweepParams& P, int64_t s, int
 // update, and neighbours are decoded once per path.
 // FP64 L = 4, 256 paths: 1.31 -> 0.93 us per sweep; FP32 with 2000 paths 9.9e10 -> 1.3e11
 // attempts/s.
-template <typename Real, class Geom, bool kOne = false>
+//
+// FP32 sums depend on their order, which is that of tm threads each taking its
+// sites in turn.  Where a launch has too few paths, or paths too large, for
+// that many threads to fill the SM (the planner's wide_threads), the path gets
+// tp > tm threads: all of them update, and in a measurement sweep the first tm
+// then add up the sums from the new spins (sum_sites).  One path per SM, half of
+// the sweeps measured: L = 10 2.5e10 -> 5.1e10 attempts/s (32 threads, now 256), L =
+// 20 1.1e11 -> 1.7e11 (160, now 512); with thermalisation alone 2.6e10 -> 9.4e10 and
+// 1.15e11 -> 2.14e11.
+// kWide paths have a body of their own: with a branch in the common one, measured
+// sweeps of the others lost 2%.
+template <typename Real, class Geom, bool kOne = false, bool kWide = false>
 __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, int sys_idx,
                                          int64_t path, const SweepParams& P, unsigned char* slice,
                                          int tid, int tp, int bar, Real* hbm_spins = nullptr) {
   using A = Arith<Real>;
+  static_assert(!kWide || (sizeof(Real) == 4 && Geom::kColumns && !kOne), "wide paths are FP32 column walks");
   Real* sp = hbm_spins ? hbm_spins : reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring));
   const int S = geo.stride();
   const uint32_t c2 = static_cast<uint32_t>(sy.path_begin + path);  // path id
@@ -1101,13 +1181,13 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
   const int64_t j_first = P.s_begin > P.n_therm ? P.s_begin - P.n_therm : 0;
   Meter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
                     reinterpret_cast<Real*>(slice + slice_red_offset()),
-                    sy.ring, tp >> 5, tid & 31, tid >> 5, tid,
+                    sy.ring, (kWide ? sy.tm : tp) >> 5, tid & 31, tid >> 5, tid,
                     1.0 / static_cast<double>(sy.N), J, hf, j_first};
   meter.start();
   unsigned char* st = path_state(P, sys_idx, path);
   Real* st_spins = st ? reinterpret_cast<Real*>(st + kStateHeader) : nullptr;
   typename Stored<Real>::C* raw = reinterpret_cast<typename Stored<Real>::C*>(sp);
-  __shared__ int cancel_flag[kMaxGroups];
+  int* const cancel_flag = cancel_flags<Real, Geom>();
   const int gidx = bar - 1;
 
   if (P.resume && st) {  // continue from the saved state
@@ -1183,7 +1263,7 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
     const PhiloxPrefix pre = philox_prefix(sw, c2, c3u, P.key);
     Partials<Real> part;
     poll_cancel(P, s, tid, &cancel_flag[gidx]);
-    if (s < P.n_therm) {
+    if (kWide || s < P.n_therm) {
       half_sweep<Real, Geom, false, false>(geo, 0, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
       group_sync(tp, bar);
       if (cancel_flag[gidx]) {
@@ -1192,28 +1272,44 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
       }
       half_sweep<Real, Geom, false, false>(geo, 1, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
       group_sync(tp, bar);
+      if constexpr (kWide) {
+        if (s >= P.n_therm) {
+          if (tid < sy.tm) {  // whole warps
+            meter.maybe_flush(s - P.n_therm);
+            const bool table = units != nullptr;
+            const int sum_K = table ? sy.sum_K : column_segments(2 * Geom::HL, kColumnChunk<Real, Geom>, sy.tm);
+            const int4* sum_units = table ? P.units + sy.sum_off : nullptr;
+            sum_sites<Geom, false>(geo, sp, tid, sy.tm, sum_K, sum_units, part);
+            sum_sites<Geom, true>(geo, sp, tid, sy.tm, sum_K, sum_units, part);
+            meter.record(part);
+          }
+          group_sync(tp, bar);
+        }
+      }
       continue;
     }
-    // Measurement sweep j.  Colour-0 sites keep their values during the
-    // colour-1 pass, so the colour-1 local fields give every bond once.
-    const int64_t j = s - P.n_therm;
-    half_sweep<Real, Geom, true, false>(geo, 0, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
-    group_sync(tp, bar);
-    if (cancel_flag[gidx]) {
-      canceled = true;
-      break;
+    if constexpr (!kWide) {
+      // Measurement sweep j.  Colour-0 sites keep their values during the
+      // colour-1 pass, so the colour-1 local fields give every bond once.
+      const int64_t j = s - P.n_therm;
+      half_sweep<Real, Geom, true, false>(geo, 0, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
+      group_sync(tp, bar);
+      if (cancel_flag[gidx]) {
+        canceled = true;
+        break;
+      }
+      meter.maybe_flush(j);
+      half_sweep<Real, Geom, true, true>(geo, 1, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
+      meter.record(part);
+      group_sync(tp, bar);
     }
-    meter.maybe_flush(j);
-    half_sweep<Real, Geom, true, true>(geo, 1, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
-    meter.record(part);
-    group_sync(tp, bar);
   }
   if (canceled) {  // the call is discarded: no record, no saved state
     group_sync(tp, bar);
     return;
   }
   const int64_t n_meas_done = P.s_end > P.n_therm ? P.s_end - P.n_therm : 0;
-  meter.finish(n_meas_done);
+  if (!kWide || (tid >> 5) < meter.nwarps) meter.finish(n_meas_done);
   group_sync(tp, bar);
 
   Real worst = Real(0);
@@ -1230,7 +1326,8 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
   }
   meter.write_record(P.records + (sy.rec_offset + path) * MP_NREC, accepted,
                      static_cast<double>(worst), P.s_end, n_meas_done, sy.N, tp, bar,
-                     accepted_before, (P.save && st) ? reinterpret_cast<double*>(st) + kAccDoubles : nullptr);
+                     accepted_before, (P.save && st) ? reinterpret_cast<double*>(st) + kAccDoubles : nullptr,
+                     kWide ? tp >> 5 : 0);
   if (P.spins != nullptr) {
     double* out = P.spins + P.spin_offset[sys_idx] + path * 3 * static_cast<int64_t>(sy.N);
     for (int c = 0; c < 2; ++c) {

@@ -15,6 +15,12 @@ __device__ __forceinline__ void dispatch_path(const DevSystem& sy, int sys_idx, 
                                               const SweepParams& P, unsigned char* slice, int tid,
                                               int tp, int bar) {
   if constexpr (kLattice > 0) {
+    if constexpr (sizeof(Real) == 4 && !kOneSite<Real, kLattice>) {
+      if (sy.tm > 0) {
+        run_path<Real, GeomSC<kLattice>, false, true>(GeomSC<kLattice>{}, sy, sys_idx, path, P, slice, tid, tp, bar);
+        return;
+      }
+    }
     run_path<Real, GeomSC<kLattice>, kOneSite<Real, kLattice>>(GeomSC<kLattice>{}, sy, sys_idx, path, P, slice, tid, tp, bar);
   } else if constexpr (kLattice == kStreamKernel || kLattice == kGlobalKernel ||
                        stream_variant_L(kLattice) > 0) {
@@ -29,6 +35,12 @@ __device__ __forceinline__ void dispatch_path(const DevSystem& sy, int sys_idx, 
     switch (sy.L) {
 #define MPK_CASE(LL)                                                           \
   case LL:                                                                     \
+    if constexpr (sizeof(Real) == 4) {                                         \
+      if (sy.tm > 0) {                                                         \
+        run_path<Real, GeomSC<LL, true>, false, true>(GeomSC<LL, true>{}, sy, sys_idx, path, P, slice, tid, tp, bar); \
+        break;                                                                 \
+      }                                                                        \
+    }                                                                          \
     run_path<Real>(GeomSC<LL, true>{}, sy, sys_idx, path, P, slice, tid, tp, bar); \
     break;
       MPK_FOR_EACH_L(MPK_CASE)
