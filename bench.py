@@ -83,8 +83,8 @@ WORKLOADS = {
         systems=[(10, 1.0, 10000)], n_therm=500, n_meas=500, precision="fp32", bound="alu",
         cpu_paths=2, ref_paths=2, fp64_paths=0, flags="random_site", order="random",
         text=("the paper's literal order, N attempts at random sites per sweep: simple cubic L=10, "
-              "J=1, h=0, T=1.0, 10^4 paths, 500+500 sweeps, FP32, one thread per path, lattices "
-              "in HBM")),
+              "J=1, h=0, T=1.0, 10^4 paths, 500+500 sweeps, FP32, one warp per path, lattices "
+              "in shared memory")),
 }
 
 LATTICES = {"sc": 0, "chain": 1, "ising": 2}

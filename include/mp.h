@@ -98,8 +98,8 @@ extern "C" {
                                  sweep is N attempts at sites drawn at random
                                  (attempt a of sweep s: counter (a, s, path,
                                  2 | sys<<8), site floor((2 r3 + 1) N / 2^33),
-                                 move from r0..r2).  One thread per path, spins
-                                 in HBM; simple-cubic and chain systems only;
+                                 move from r0..r2).  One warp per path (a thread
+                                 for the smallest); simple-cubic and chain systems only;
                                  mp_run_sweeps, mp_checkpoint and mp_restore
                                  return MP_EINVAL */
 #define MP_FLAG_TEST_STALL 0x100u /* failure injection for tests: streamed paths
@@ -358,7 +358,8 @@ int mp_restore(mp_handle h, const void* buf, size_t nbytes);
  * run is in flight. */
 int mp_cancel(mp_handle h);
 
-/* Launch shape of one system: threads per path, paths per CTA, and where
+/* Launch shape of one system: threads per path (FP32 simple cubic: those that
+ * order a path's sums; by default the launch may have more), paths per CTA, and where
  * its lattice lives during a run: 0 in one CTA's shared memory, 1 streamed
  * from HBM through shared-memory half-plane buffers, 2 split over the shared
  * memory of the two CTAs of a cluster (FP32 simple cubic L = 32: each CTA
