@@ -191,6 +191,28 @@ __host__ __device__ inline int4 column_unit(int L, int K, int u) {
   return d;
 }
 
+// ----------------------------------------------------- streamed rows --
+// Row k = 0 .. 3 of a streamed lattice's thread whose first row is y0 and whose
+// rows lie RS apart (3 RS <= L <= 4 RS, y0 < RS): where it starts in the
+// half-plane, relative to row y0, and the offsets to its +-y neighbours
+// (periodic).  The fourth row may lie outside the lattice: then it stands for
+// row y0 (with that row's neighbours) and is not `act`ed on.  With k a constant
+// all but the first row's -y and the last two rows' +y are constants too.
+struct StreamRow {
+  int off, yp, ym;
+  bool act;
+};
+__host__ __device__ inline StreamRow stream_row(int L, int RS, int y0, int k) {
+  const int HL = L / 2;
+  const bool act = k < 3 || y0 + 3 * RS < L;
+  StreamRow r;
+  r.act = act;
+  r.off = act ? k * (HL * RS) : 0;
+  r.yp = (k >= 2 && y0 + k * RS == L - 1) ? -(L - 1) * HL : HL;
+  r.ym = ((k == 0 || !act) && y0 == 0) ? (L - 1) * HL : -HL;
+  return r;
+}
+
 constexpr int kErrTimeout = 1;
 constexpr int kErrCanceled = 2;
 constexpr int kErrLaunch = 3;  // paths for two-CTA clusters in a launch without clusters

@@ -1817,10 +1817,11 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   constexpr bool kFixedRows = kL > 0 && kRS > 0 && kL % kRS == 0;
   // FP32 with three or four rows per thread (the planner's layouts): see phase
   constexpr bool kFourRows = sizeof(Real) == 4 && kRS == 0;
-  const bool four_rows = 3 * RS <= L && L <= 4 * RS, fourth = y0 + 3 * RS < L;
+  const bool four_rows = 3 * RS <= L && L <= 4 * RS;
   const int hp0 = hx + HL * y0;
-  const int ym0 = y0 == 0 ? (L - 1) * HL : -HL;  // rows that may wrap in y: the first and the last
-  const int yp2 = y0 + 2 * RS == L - 1 ? -(L - 1) * HL : HL, yp3 = y0 + 3 * RS == L - 1 ? -(L - 1) * HL : HL;
+  StreamRow srow[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) srow[k] = stream_row(L, RS, y0, k);
   int accepted = 0;
   bool ok = true;
 
@@ -1913,7 +1914,7 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
         if constexpr (kFourRows) {
           if (!active) return;
           // Rows y0 + k RS, k = 0 .. 3, the fourth only where it lies in the
-          // lattice (act): offsets, parities and wraps once per thread, no
+          // lattice (act; stream_row): offsets, parities and wraps once per thread, no
           // branch between the rows, whose Philox chains the compiler interleaves.
           const int pz = (y0 + z + c) & 1;
           const int xoa = pz ? oxp1 : oxm0, xob = pz ? oxm0 : oxp1;
@@ -1921,10 +1922,10 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
           auto rows = [&](auto meas_c, auto energy_c) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              const bool act = k < 3 || fourth;
-              const int hp = hp0 + (act ? k * (HL * RS) : 0);
+              const bool act = srow[k].act;
+              const int hp = hp0 + srow[k].off;
               const int xo = hp + (k & 1 ? xoc : xoa), p = k & 1 ? pc : pz;
-              const int yp = hp + (k == 3 ? yp3 : k == 2 ? yp2 : HL), ym = hp + (k == 0 ? ym0 : -HL);
+              const int yp = hp + srow[k].yp, ym = hp + srow[k].ym;
               const V3<Real> f = add3(add3(add3(add3(add3(same.ld(hp), same.ld(xo)), same.ld(yp)), same.ld(ym)),
                                            up.ld(hp)), dn.ld(hp));
               update_spin<decltype(meas_c)::value, decltype(energy_c)::value>(
