@@ -573,7 +573,9 @@ __device__ __forceinline__ void update(uint32_t i, const PhiloxPrefix& pre, cons
   }
 }
 
-// One-site form (see run_path): a move drawn ahead of its update.
+// One-site form (see run_path): a move drawn ahead of its update.  A thread
+// without a site (act = false) reads no spin of the colour that the others are
+// writing.
 template <typename Real>
 struct Ahead;
 template <>
@@ -584,7 +586,9 @@ struct Ahead<float> {
   template <bool kMeas, bool kEnergy>
   __device__ __forceinline__ void apply(const SpinView<float>& own, int hh, V3<float> f, const Couplings<float>& cp,
                                         bool act, int& accepted, Partials<float>& part) const {
-    settle<kMeas, kEnergy>(t, r2, own, hh, own.ld(hh), f, cp, act, accepted, part);
+    V3<float> a{};
+    if (act) a = own.ld(hh);
+    settle<kMeas, kEnergy>(t, r2, own, hh, a, f, cp, act, accepted, part);
   }
 };
 template <>
@@ -600,10 +604,11 @@ struct Ahead<double> {
   template <bool kMeas, bool kEnergy>
   __device__ __forceinline__ void apply(const SpinView<double>& own, int hh, V3<double> f, const Couplings<double>& cp,
                                         bool act, int& accepted, Partials<double>& part) const {
-    const V3<double> a = own.ld(hh);
+    V3<double> a{};
+    if (act) a = own.ld(hh);
     bool ok, open;
     fix_test(d, a, f, cp, ok, open);
-    if (open) ok = accept_exact(t.x - a.x, t.y - a.y, t.z - a.z, f.x, f.y, f.z, cp.sys, r2);
+    if (open && act) ok = accept_exact(t.x - a.x, t.y - a.y, t.z - a.z, f.x, f.y, f.z, cp.sys, r2);
     ok = ok && act;
     const V3<double> n = ok ? V3<double>{t.x, t.y, t.z} : a;
     if (ok) {
