@@ -198,12 +198,6 @@ struct mp_state {
   cudaGraphExec_t gexec = nullptr;
   bool graph_dirty = true;
   bool launched = false;           // mp_run has run with the current seed (a graph is made from the second run on)
-  // estimates and error word of the last run, read together (mp_estimates)
-  std::vector<double> est_host;
-  uint64_t runs = 0, est_run = 0;  // runs queued; the run est_host holds
-  double est_elapsed = 0.0;
-  int est_error = 0;
-  bool est_exposed = false;        // the caller has the estimates' device pointer
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
   bool ran = false;
   std::string err;
@@ -1235,7 +1229,6 @@ int mp_run(mp_handle h) {
     direct = cs == cudaStreamCaptureStatusNone;
     h->launched = direct;
   }
-  ++h->runs;
   if (direct) {
     *h->h_cancel = 0;
     int rc = enqueue_run(h, 0, h->n_therm + h->n_meas, false, false);
@@ -1284,33 +1277,27 @@ int mp_estimates(mp_handle h, int system, mp_estimates_t* out) {
     return fail(h, MP_EINVAL, "bad system index %d or NULL output", system);
   if (!h->ran) return fail(h, MP_ESTATE, "no run yet");
   DeviceGuard dg(h->device);
-  // Every system's estimates of a run and its error word come in one copy
-  // (they lie side by side), 29 us saved for each system after the first.  Not
-  // once the caller has their device pointer and may write through it.
-  const size_t n = h->hsys.size(), count = n * MP_NEST + 1;
-  if (n > 1024 || h->est_exposed) {
-    MP_CUDA(h, cudaMemcpyAsync(out, h->d_est + static_cast<int64_t>(system) * MP_NEST,
-                               sizeof(mp_estimates_t), cudaMemcpyDeviceToHost, h->stream));
-    MP_CUDA(h, cudaStreamSynchronize(h->stream));
-    float ms = 0.f;  // sweep and reduction kernels of the last run
-    out->elapsed_s = cudaEventElapsedTime(&ms, h->ev[0], h->ev[2]) == cudaSuccess ? 1e-3 * ms : NAN;
-    cudaGetLastError();
-    return check_error_flag(h);
+  // Read from the device on every call: the run may have been replayed from a
+  // graph of the caller's, which this side does not see.  The estimates lie
+  // before the error word, so where few systems are in between one copy brings
+  // both (each copy to pageable memory costs about 15 us).
+  double buf[512];
+  const size_t count = (h->hsys.size() - system) * MP_NEST + 1;
+  const double* d_row = h->d_est + static_cast<int64_t>(system) * MP_NEST;
+  int flag = 0;
+  if (count <= 512) {
+    MP_CUDA(h, cudaMemcpyAsync(buf, d_row, sizeof(double) * count, cudaMemcpyDeviceToHost, h->stream));
+  } else {
+    MP_CUDA(h, cudaMemcpyAsync(buf, d_row, sizeof(mp_estimates_t), cudaMemcpyDeviceToHost, h->stream));
+    MP_CUDA(h, cudaMemcpyAsync(&flag, h->d_error, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   }
-  if (h->est_run != h->runs) {
-    h->est_host.resize(count);
-    h->est_run = 0;
-    MP_CUDA(h, cudaMemcpyAsync(h->est_host.data(), h->d_est, sizeof(double) * count, cudaMemcpyDeviceToHost, h->stream));
-    MP_CUDA(h, cudaStreamSynchronize(h->stream));
-    float ms = 0.f;
-    h->est_elapsed = cudaEventElapsedTime(&ms, h->ev[0], h->ev[2]) == cudaSuccess ? 1e-3 * ms : NAN;
-    cudaGetLastError();
-    std::memcpy(&h->est_error, &h->est_host[n * MP_NEST], sizeof(int));
-    h->est_run = h->runs;
-  }
-  std::memcpy(out, &h->est_host[static_cast<size_t>(system) * MP_NEST], sizeof(mp_estimates_t));
-  out->elapsed_s = h->est_elapsed;
-  return error_status(h, h->est_error);
+  MP_CUDA(h, cudaStreamSynchronize(h->stream));
+  if (count <= 512) std::memcpy(&flag, &buf[count - 1], sizeof(int));
+  std::memcpy(out, buf, sizeof(mp_estimates_t));
+  float ms = 0.f;  // sweep and reduction kernels of the last run
+  out->elapsed_s = cudaEventElapsedTime(&ms, h->ev[0], h->ev[2]) == cudaSuccess ? 1e-3 * ms : NAN;
+  cudaGetLastError();
+  return error_status(h, flag);
 }
 
 int mp_paths(mp_handle h, int system, double* host_out, int64_t cap) {
@@ -1331,10 +1318,7 @@ int mp_paths(mp_handle h, int system, double* host_out, int64_t cap) {
 int mp_device_buffers(mp_handle h, double** d_records, double** d_estimates) {
   if (!h) return fail(nullptr, MP_EINVAL, "handle is NULL");
   if (d_records) *d_records = h->d_rec;
-  if (d_estimates) {
-    *d_estimates = h->d_est;
-    h->est_exposed = true;
-  }
+  if (d_estimates) *d_estimates = h->d_est;
   return MP_OK;
 }
 
@@ -1485,7 +1469,6 @@ int mp_run_sweeps(mp_handle h, int64_t n_sweeps) {
   if (rc != MP_OK) return rc;
   const int64_t s_end = std::min(total, h->sweeps_done + n_sweeps);
   *h->h_cancel = 0;
-  ++h->runs;
   rc = enqueue_run(h, h->sweeps_done, s_end, h->sweeps_done > 0, true);
   if (rc != MP_OK) return rc;
   MP_CUDA(h, cudaStreamSynchronize(h->stream));
