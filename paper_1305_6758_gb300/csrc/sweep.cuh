@@ -426,7 +426,7 @@ template <>
 struct Couplings<double> {
   const DevSystem* sys;
   float cj, ch;    // log2 of the acceptance is cj d.h + ch d_z, d and h in units of 2^-28
-  float lo, hi;    // 1 -+ the bound on the relative error of the FP32 acceptance
+  float lo, hi;    // 1 -+ the bound on the relative error of the FP32 acceptance (0 and infinity: none)
   __device__ explicit Couplings(const DevSystem* s) : sys(s) {
     const double bj = s->beta * s->J, bh = s->beta * s->h;
     cj = static_cast<float>(bj * 1.4426950408889634 * 0x1p-56);
@@ -435,10 +435,13 @@ struct Couplings<double> {
     // (2^-21.2 of the hardware sine and cosine, 2^-23 of their argument, 2^-22
     // of the radius), d by 1.5e-6, h by 3.7e-7, so d.h by 1.9e-5; the exponent's
     // own roundings are 2^-21 of at most 33 (beyond that the test is decided),
-    // ex2 and the uniform add 2^-22.  Taken a third larger.
+    // ex2 and the uniform add 2^-22.  Taken a third larger, which covers
+    // exp(+-bound) - 1, the error of the acceptance, while it is below 1/4.  Beyond
+    // that (beta |J| = 1e4) no move is decided here: nothing is below 0, and
+    // nothing above p times infinity (a p of 0 makes it NaN).
     const float tol = static_cast<float>(2.5e-5 * fabs(bj) + 3e-6 * fabs(bh) + 2e-5);
-    lo = 1.0f - tol;
-    hi = 1.0f + tol;
+    lo = tol < 0.25f ? 1.0f - tol : 0.0f;
+    hi = tol < 0.25f ? 1.0f + tol : __int_as_float(0x7f800000);
   }
 };
 
