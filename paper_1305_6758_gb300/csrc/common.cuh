@@ -21,7 +21,10 @@ __host__ __device__ inline int path_init_mode(int32_t mode, int64_t path, int64_
 }
 
 constexpr int kAccDoubles = 24;      // FP64 per-path accumulators (>= MP_NREC) in shared memory
-constexpr int kRedSlots = 4;         // doubles per warp in the per-sweep reduction
+constexpr int kRedSlots = 4;         // partial sums per warp in the per-sweep reduction
+// Their bytes in shared memory: numbers of up to 8 bytes, or (FP64 form)
+// 96-bit integers.
+constexpr int kRedBytes = kRedSlots * 8, kRedBytesFix = kRedSlots * 12;
 constexpr int kMaxCta = 1024;
 // Most paths one CTA can hold: one warp each (groups of more than one warp
 // are limited to 15 by the named barriers 1..15).
@@ -221,12 +224,12 @@ constexpr int kCancelPoll = 16;    // sweeps between polls of the cancel flag
 
 // Byte offsets inside one path's shared-memory slice.
 // [acc: FP64 accumulators][ring: 2 x R sweeps x warps x kRedSlots partials][spins]
-// (ring elements are sized 8 bytes, enough for either precision and for the
-// two doubles per warp of the final reduction)
+// (a ring element has `red` bytes, kRedBytes or kRedBytesFix, enough for the
+// two doubles per warp of the final reduction too)
 __host__ __device__ constexpr int slice_acc_offset() { return 0; }
 __host__ __device__ constexpr int slice_red_offset() { return kAccDoubles * 8; }
-__host__ __device__ inline int slice_spin_offset(int tp, int ring) {
-  return kAccDoubles * 8 + (2 * ring * (tp / 32) * kRedSlots * 8 + 127) / 128 * 128;
+__host__ __device__ inline int slice_spin_offset(int tp, int ring, int red) {
+  return kAccDoubles * 8 + (2 * ring * (tp / 32) * red + 127) / 128 * 128;
 }
 
 }  // namespace mpk

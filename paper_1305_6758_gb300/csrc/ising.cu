@@ -170,7 +170,7 @@ __device__ void run_path_ising(const DevSystem& sy, int sys_idx, int64_t path,
   const int L = sy.L, N = sy.N, NH = sy.NH;
   const StripWalk walk(L, tp, ising_segment(L, tp));
   const int HL = walk.HL;
-  unsigned char* base = slice + slice_spin_offset(tp, sy.ring);
+  unsigned char* base = slice + slice_spin_offset(tp, sy.ring, kRedBytes);
   unsigned char* table_at = base + ((128u - (smem_addr(base) & 127u)) & 127u);
   uint32_t* sp = reinterpret_cast<uint32_t*>(base + kIsingThrBytes);  // strips of colour 0, then of colour 1
   const uint32_t c2 = static_cast<uint32_t>(sy.path_begin + path);  // path id
@@ -339,7 +339,7 @@ int ising_threads(int L, int64_t paths_per_sm, int smem_max, int ring) {
   double best = -1.0;
   int best_t = 32;
   for (int t = 32; t <= kIsingThreads && (t == 32 || t < 2 * S); t += 32) {
-    const int slice = (slice_spin_offset(t, ring) + ising_slice_spin_bytes(L) + 127) / 128 * 128;
+    const int slice = (slice_spin_offset(t, ring, kRedBytes) + ising_slice_spin_bytes(L) + 127) / 128 * 128;
     int64_t fit = std::min<int64_t>(smem_max / slice, t > 32 ? std::min(15, kIsingThreads / t) : kIsingThreads / t);
     fit = std::min(fit, paths_per_sm);
     if (fit < 1) continue;

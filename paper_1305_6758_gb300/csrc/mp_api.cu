@@ -12,6 +12,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <string>
@@ -107,6 +108,11 @@ void ising_thresholds(const mp_system& s, unsigned long long* t) {
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
+// Bytes of a path's partial sums per warp and measurement sweep.
+int meter_bytes(const mp_system& s, int precision) {
+  return precision == MP_FP64 && s.lattice != MP_LATTICE_ISING ? kRedBytesFix : kRedBytes;
+}
+
 // Streamed lattices: one half-plane (one colour of one z-plane, 3 L^2/2 values)
 // padded to 16 bytes, in bytes.
 int half_plane_bytes(int L, int real) { return round_up(3 * (L * L / 2) * real, 16); }
@@ -133,7 +139,7 @@ bool streamed(const mp_system& s, int precision, uint32_t flags) {
 bool in_place(const mp_system& s, int precision, uint32_t flags, int optin) {
   if (!streamed(s, precision, flags)) return false;
   const int real = precision == MP_FP64 ? 8 : 4;
-  return 128 + 9 * half_plane_bytes(s.L, real) + slice_spin_offset(32, 1) > optin - 4096;
+  return 128 + 9 * half_plane_bytes(s.L, real) + slice_spin_offset(32, 1, meter_bytes(s, precision)) > optin - 4096;
 }
 
 }  // namespace
@@ -467,7 +473,7 @@ int plan(mp_state* h, const mp_config* cfg) {
     const int64_t load = (batch_paths + sms - 1) / sms;  // paths per SM
     double best = 0.0;
     for (int c = tp[k]; c <= std::min(cta_max, round_up(NH, 32)); c += 32) {
-      const int s = round_up(slice_spin_offset(c, ring[k]) + static_cast<int>(lat), 128);
+      const int s = round_up(slice_spin_offset(c, ring[k], kRedBytes) + static_cast<int>(lat), 128);
       int64_t fit = std::min<int64_t>(smem_max / s, c > 32 ? std::min(15, cta_max / c) : cta_max / c);
       fit = std::min(fit, load);
       if (fit < 1) continue;
@@ -498,6 +504,7 @@ int plan(mp_state* h, const mp_config* cfg) {
   for (int k = 0; k < n; ++k) {
     const int64_t N = sites_of(h->systems[k]);
     const int NH = static_cast<int>((N + 1) / 2);
+    const int red = meter_bytes(h->systems[k], h->precision);
     int t = (static_cast<int>(h->tp_override.size()) > k && h->tp_override[k] > 0) ? h->tp_override[k]
                                                                                   : cfg->threads_per_path;
     const bool by_default = t == 0;
@@ -510,7 +517,7 @@ int plan(mp_state* h, const mp_config* cfg) {
       ring[k] = 16;
       // the ring of the CTA that owns the path holds both CTAs' warps
       auto need = [&]() {
-        return round_up(slice_spin_offset(2 * cta_max, ring[k]) + pair_spin_bytes(kPairL, real), 128);
+        return round_up(slice_spin_offset(2 * cta_max, ring[k], red) + pair_spin_bytes(kPairL, real), 128);
       };
       pick_ring(ring[k], slice[k], need, cta_max);
       if (slice[k] > smem_max)
@@ -525,7 +532,7 @@ int plan(mp_state* h, const mp_config* cfg) {
       if (t > cta_max) return fail(h, MP_EINVAL, "threads_per_path %d above %d", t, cta_max);
       tp[k] = t;
       ring[k] = 16;
-      pick_ring(ring[k], slice[k], [&]() { return round_up(slice_spin_offset(t, ring[k]), 128); }, t);
+      pick_ring(ring[k], slice[k], [&]() { return round_up(slice_spin_offset(t, ring[k], red), 128); }, t);
       max_tp = std::max(max_tp, t);
       continue;
     }
@@ -538,7 +545,7 @@ int plan(mp_state* h, const mp_config* cfg) {
       tp[k] = t;
       ring[k] = 16;
       auto need = [&]() {
-        return round_up(slice_spin_offset(t, ring[k]) + 128 + 9 * half_plane_bytes(L, real), 128);
+        return round_up(slice_spin_offset(t, ring[k], red) + 128 + 9 * half_plane_bytes(L, real), 128);
       };
       pick_ring(ring[k], slice[k], need, t);
       if (slice[k] > smem_max)
@@ -547,29 +554,43 @@ int plan(mp_state* h, const mp_config* cfg) {
       max_tp = std::max(max_tp, t);
       continue;
     }
-    if (t == 0 && h->systems[k].lattice == MP_LATTICE_ISING)
-      t = ising_threads(h->systems[k].L, (batch_paths + sms - 1) / sms, smem_max, 16);
-    if (t == 0 && h->systems[k].lattice == MP_LATTICE_SC && real == 8) {
-      // FP64 form: its sums are exact, so the layout is free, and its lattices
-      // are large (L = 16: two paths per SM): the count that fills its own
-      // lanes best, weighed with the warps the SM then holds (of 16).  L = 16,
-      // 3072 paths: 6.2e10 attempts/s with 128 threads, 7.3e10 with 256; L = 20,
+    // shared-memory bytes of the lattice, and of a path of t threads
+    const int64_t lat = h->systems[k].lattice == MP_LATTICE_ISING ? ising_slice_spin_bytes(h->systems[k].L)
+                                                                   : lattice_bytes(h->systems[k], real);
+    auto need_of = [&](int threads, int r) {
+      return static_cast<int>(std::min<int64_t>(INT32_MAX / 2, round_up(slice_spin_offset(threads, r, red) + lat, 128)));
+    };
+    // Ising and the FP64 form: a path's sums are exact, so its record does not
+    // depend on the number of threads, which is chosen by the paths that an SM
+    // gets; it does depend on the ring (the sweeps summed together), which is
+    // therefore that of the threads chosen for a full GPU.
+    std::function<int(int64_t, int)> by_load;  // threads for so many paths per SM and this ring
+    if (h->systems[k].lattice == MP_LATTICE_ISING) {
+      by_load = [&](int64_t per_sm, int r) { return ising_threads(h->systems[k].L, per_sm, smem_max, r); };
+    } else if (h->systems[k].lattice == MP_LATTICE_SC && real == 8) {
+      // FP64 lattices are large (L = 16: two paths per SM): the count that fills
+      // its own lanes best, weighed with the warps the SM then holds (of 16).  L =
+      // 16, 3072 paths: 6.2e10 attempts/s with 128 threads, 7.3e10 with 256; L = 20,
       // 500 paths: 3.4e10 with 160, 6.2e10 with 512.
-      double best = -1.0;
-      for (int c = 32; c <= std::min(cta_max, round_up(NH, 32)); c += 32) {
-        const int units = h->systems[k].L * h->systems[k].L / 2 * column_segments(h->systems[k].L, 1, c);
-        const int s = round_up(slice_spin_offset(c, 1) + static_cast<int>(lattice_bytes(h->systems[k], real)), 128);
-        int64_t fit = std::min<int64_t>(smem_max / s, c > 32 ? std::min(15, cta_max / c) : cta_max / c);
-        fit = std::min(fit, (batch_paths + sms - 1) / sms);
-        if (fit < 1) continue;
-        const double rate = units / (static_cast<double>((units + c - 1) / c) * c) *
-                            std::min(1.0, static_cast<double>(fit) * c / 512.0);
-        if (rate > best + 1e-9) {
-          best = rate;
-          t = c;
+      by_load = [&](int64_t per_sm, int r) {
+        double best = -1.0;
+        int best_t = 0;
+        for (int c = 32; c <= std::min(cta_max, round_up(NH, 32)); c += 32) {
+          const int units = h->systems[k].L * h->systems[k].L / 2 * column_segments(h->systems[k].L, 1, c);
+          int64_t fit = std::min<int64_t>(smem_max / need_of(c, r), c > 32 ? std::min(15, cta_max / c) : cta_max / c);
+          fit = std::min(fit, per_sm);
+          if (fit < 1) continue;
+          const double rate = units / (static_cast<double>((units + c - 1) / c) * c) *
+                              std::min(1.0, static_cast<double>(fit) * c / 512.0);
+          if (rate > best + 1e-9) {
+            best = rate;
+            best_t = c;
+          }
         }
-      }
+        return best_t;
+      };
     }
+    if (t == 0 && by_load) t = by_load(INT64_MAX, h->systems[k].lattice == MP_LATTICE_ISING ? 16 : 1);
     if (t == 0 && h->systems[k].lattice == MP_LATTICE_SC) {
       // a divisor of the sites per colour lets each thread walk a block of
       // columns; pick the one closest to the target sites per thread
@@ -586,15 +607,17 @@ int plan(mp_state* h, const mp_config* cfg) {
     if (t == 0)
       t = std::min(cta_max, std::max(32, round_up(static_cast<int>(std::ceil(NH / target)), 32)));
     if (t > cta_max) return fail(h, MP_EINVAL, "threads_per_path %d above %d", t, cta_max);
-    tp[k] = t;
     // partial-sum ring: the largest power of two up to 16 sweeps that fits
     ring[k] = 16;
-    // shared-memory bytes of the lattice
-    const int64_t lat = h->systems[k].lattice == MP_LATTICE_ISING ? ising_slice_spin_bytes(h->systems[k].L)
-                                                                   : lattice_bytes(h->systems[k], real);
-    pick_ring(ring[k], slice[k], [&]() {
-      return static_cast<int>(std::min<int64_t>(INT32_MAX / 2, round_up(slice_spin_offset(t, ring[k]) + lat, 128)));
-    }, t);
+    pick_ring(ring[k], slice[k], [&]() { return need_of(t, ring[k]); }, t);
+    if (by_default && by_load) {
+      const int loaded = by_load((batch_paths + sms - 1) / sms, ring[k]);
+      if (loaded > 0) {
+        t = loaded;
+        slice[k] = need_of(t, ring[k]);
+      }
+    }
+    tp[k] = t;
     if (slice[k] > smem_max)
       return fail(h, MP_EINVAL, "system %d needs %d bytes of shared memory per path (max %d)", k,
                   slice[k], smem_max);

@@ -878,7 +878,11 @@ __device__ __forceinline__ void sum_sites(const Geom& geo, const float* sp, int 
 // R sweeps is flushed into the FP64 accumulators by all warps together after
 // the next barrier while the other half fills, so no warp carries the
 // bookkeeping alone and no FP64 operation runs per sweep.
-template <typename Real>
+// kFix (FP64 form): the partial sums are 96-bit integers, added up exactly over
+// the warps and rounded once, so that a path's record does not depend on how
+// many threads ran it: the planner chooses them by the paths per SM, and
+// processes that each run a part of an ensemble reproduce one that runs all.
+template <typename Real, bool kFix = false>
 struct Meter {
   double* acc;
   Real* red;
@@ -900,37 +904,63 @@ struct Meter {
     if (nslot == 0) nslot = nwarps;
     cur = static_cast<int>(((j_first / R) & 1) * R + j_first % R);
   }
-  __device__ Real* slot(int64_t j) const {
-    return red + ((((j / R) & 1) * R + (j % R)) * nslot) * kRedSlots;
+  // first of the kRedSlots partial sums of ring slot q
+  __device__ Real* at(int q) const { return red + (q * nslot) * kRedSlots; }
+  __device__ int slot(int64_t j) const { return static_cast<int>(((j / R) & 1) * R + (j % R)); }
+  __device__ Real* cur_slot() const { return at(cur); }
+  // the same of warp w, as words (kFix)
+  __device__ uint32_t* words(int q, int w) const {
+    return reinterpret_cast<uint32_t*>(red) + (q * nslot + w) * (kRedBytesFix / 4);
   }
-  __device__ Real* cur_slot() const { return red + (cur * nslot) * kRedSlots; }
   __device__ void advance() {
     if (++cur == 2 * R) cur = 0;
   }
   // Per-site observables (Sec. 2.2) of one measurement sweep from its slot.
-  __device__ void observe(const Real* sl, Real& e, Real& ex, Real& ey, Real& ez) const {
+  __device__ void observe(int q, Real& e, Real& ex, Real& ey, Real& ez) const {
     Real E = Real(0), MX = Real(0), MY = Real(0), MZ = Real(0);
-    for (int w = 0; w < nslot; ++w) {
-      E += sl[w * kRedSlots + 0];
-      MX += sl[w * kRedSlots + 1];
-      MY += sl[w * kRedSlots + 2];
-      MZ += sl[w * kRedSlots + 3];
+    if constexpr (kFix) {
+      Wide wE, wX, wY, wZ;
+      for (int w = 0; w < nslot; ++w) {
+        const uint4* p = reinterpret_cast<const uint4*>(words(q, w));
+        const uint4 a = p[0], b = p[1], c = p[2];
+        wE.add(a.x, a.y, a.z);
+        wX.add(a.w, b.x, b.y);
+        wY.add(b.z, b.w, c.x);
+        wZ.add(c.y, c.z, c.w);
+      }
+      E = wE.real(kEnergyBits);
+      MX = wX.real(kFixBits);
+      MY = wY.real(kFixBits);
+      MZ = wZ.real(kFixBits);
+    } else {
+      const Real* sl = at(q);
+      for (int w = 0; w < nslot; ++w) {
+        E += sl[w * kRedSlots + 0];
+        MX += sl[w * kRedSlots + 1];
+        MY += sl[w * kRedSlots + 2];
+        MZ += sl[w * kRedSlots + 3];
+      }
     }
     const Real rN = static_cast<Real>(invN);
-    e = (-J * E - hf * MZ) * rN;
+    // (FP64: roundings spelled out, for the same record from either flush)
+    if constexpr (sizeof(Real) == 8) e = __dmul_rn(__fma_rn(-J, E, __dmul_rn(-hf, MZ)), rN);
+    else e = (-J * E - hf * MZ) * rN;
     ex = MX * rN;
     ey = MY * rN;
     ez = MZ * rN;
   }
   // Store this warp's partials of the current measurement sweep and move to
   // the next (every lane calls, once per measurement sweep, in order).
-  // FP64 form: the warp's sums are exact integers; lane k < 4 rounds sum k.
+  // FP64 form: exact integers, three words each.
   __device__ void record(Partials<double> part) {
     // lanes 0 .. 3: E, M_y, M_x, M_z
     const Wide v = warp_sums(part.eb, part.mx, part.my, part.mz, lane);
-    if (lane < 4)
-      (cur_slot() + (slot_off + warp) * kRedSlots)[lane == 1 ? 2 : lane == 2 ? 1 : lane] =
-          v.real(lane == 0 ? kEnergyBits : kFixBits);
+    if (lane < 4) {
+      uint32_t* r = words(cur, slot_off + warp) + 3 * (lane == 1 ? 2 : lane == 2 ? 1 : lane);
+      r[0] = v.w0;
+      r[1] = v.w1;
+      r[2] = v.w2;
+    }
     advance();
   }
   __device__ void record(Partials<float> part) {
@@ -951,10 +981,15 @@ struct Meter {
     }
     advance();
   }
+  // a b, rounded by itself in FP64 (whatever is added to it later).
+  static __device__ __forceinline__ Real product(Real a, Real b) {
+    if constexpr (sizeof(Real) == 8) return __dmul_rn(a, b);
+    else return a * b;
+  }
   // The same by one warp in a third of the FP64 instructions (76 cycles each,
   // and a small lattice's flush is a good part of its sweeps): lanes l and
   // l + 16 take sweep j0 + l, each half of the observables, and the 16 sweeps
-  // are summed by exchanges that halve what a lane carries.
+  // are summed by exchanges that halve what a lane carries, in flush's order.
   __device__ void flush_warp(int64_t j0, int n) const {
     Real e = Real(0), ex = Real(0), ey = Real(0), ez = Real(0);
     const int l = lane & 15;
@@ -965,11 +1000,11 @@ struct Meter {
     Real v[8];
     const Real p = upper ? ez : e;
     v[0] = p;
-    v[1] = p * p;
+    v[1] = product(p, p);
     v[2] = upper ? fabs(ez) : m;
-    v[3] = upper ? e * m : m2;
-    v[4] = upper ? e * ez : m2 * m2;
-    v[5] = upper ? m * ez : ex;
+    v[3] = upper ? product(e, m) : m2;
+    v[4] = upper ? product(e, ez) : product(m2, m2);
+    v[5] = upper ? product(m, ez) : ex;
     v[6] = upper ? Real(0) : ey;
     v[7] = Real(0);
 #pragma unroll
@@ -1008,22 +1043,25 @@ struct Meter {
       Real v;
       switch (k) {  // k is the same in every lane of the warp
         case MP_R_E: v = e; break;
-        case MP_R_E2: v = e * e; break;
+        case MP_R_E2: v = product(e, e); break;
         case MP_R_M: v = m; break;
         case MP_R_M2: v = m2; break;
-        case MP_R_M4: v = m2 * m2; break;
+        case MP_R_M4: v = product(m2, m2); break;
         case MP_R_MX: v = ex; break;
         case MP_R_MY: v = ey; break;
         case MP_R_MZ: v = ez; break;
-        case MP_R_MZ2: v = ez * ez; break;
+        case MP_R_MZ2: v = product(ez, ez); break;
         case MP_R_AMZ: v = fabs(ez); break;
-        case MP_R_EM: v = e * m; break;
-        case MP_R_EMZ: v = e * ez; break;
-        default: v = m * ez; break;  // MP_R_MMZ
+        case MP_R_EM: v = product(e, m); break;
+        case MP_R_EMZ: v = product(e, ez); break;
+        default: v = product(m, ez); break;  // MP_R_MMZ
       }
       if (lane >= n) v = Real(0);
+      // FP64: in flush_warp's order (a path of one warp may take either)
+      constexpr int kOrder[2][5] = {{16, 8, 4, 2, 1}, {16, 4, 2, 1, 8}};
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
+      for (int q = 0; q < 5; ++q) {
+        const int o = kOrder[sizeof(Real) == 8][q];
         if (o < R) v += A::shfl(v, o);
       }
       if (lane == 0) acc[k] += static_cast<double>(v);
@@ -1088,6 +1126,12 @@ struct Meter {
     }
   }
 };
+
+// The measurement state of the Heisenberg kernels and its bytes per warp and sweep.
+template <typename Real>
+using PathMeter = Meter<Real, sizeof(Real) == 8>;
+template <typename Real>
+constexpr int kMeterBytes = sizeof(Real) == 8 ? kRedBytesFix : kRedBytes;
 
 // Initial spin of site i: uniform on the sphere (Sec. 2.2), uniform angles,
 // or the ordered start of Sec. 5.
@@ -1161,7 +1205,7 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
                                          int tid, int tp, int bar, Real* hbm_spins = nullptr) {
   using A = Arith<Real>;
   static_assert(!kWide || (sizeof(Real) == 4 && Geom::kColumns && !kOne), "wide paths are FP32 column walks");
-  Real* sp = hbm_spins ? hbm_spins : reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring));
+  Real* sp = hbm_spins ? hbm_spins : reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring, kMeterBytes<Real>));
   const int S = geo.stride();
   const uint32_t c2 = static_cast<uint32_t>(sy.path_begin + path);  // path id
   const uint32_t c3u = kTagUpdate | (static_cast<uint32_t>(sys_idx) << 8);
@@ -1187,7 +1231,7 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
     }
   }
   const int64_t j_first = P.s_begin > P.n_therm ? P.s_begin - P.n_therm : 0;
-  Meter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
+  PathMeter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
                     reinterpret_cast<Real*>(slice + slice_red_offset()),
                     sy.ring, (kWide ? sy.tm : tp) >> 5, tid & 31, tid >> 5, tid,
                     1.0 / static_cast<double>(sy.N), J, hf, j_first};
@@ -1468,7 +1512,7 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
   constexpr int HL = G::HL, HP = G::HP, ZL = G::ZL, S = G::S;
   constexpr int NH = L * L * L / 2;  // sites per colour of the whole lattice
   // rank 0's ring holds the partials of both CTAs' warps
-  Real* sp = reinterpret_cast<Real*>(slice + slice_spin_offset(2 * tp, sy.ring));
+  Real* sp = reinterpret_cast<Real*>(slice + slice_spin_offset(2 * tp, sy.ring, kMeterBytes<Real>));
   Real* partner_sp = map_rank(sp, rank ^ 1u);
   const int zbase = static_cast<int>(rank) * ZL;
   const uint32_t c2 = static_cast<uint32_t>(sy.path_begin + path);  // path id
@@ -1479,7 +1523,7 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
   const Couplings<Real> cp(P.systems + sys_idx);
   const int64_t j_first = P.s_begin > P.n_therm ? P.s_begin - P.n_therm : 0;
   Real* red0 = reinterpret_cast<Real*>(slice + slice_red_offset());
-  Meter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
+  PathMeter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
                     rank == 0 ? red0 : map_rank(red0, 0u),
                     sy.ring, tp >> 5, tid & 31, tid >> 5, tid,
                     1.0 / static_cast<double>(sy.N), J, hf, j_first};
@@ -1733,9 +1777,9 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   const int hps = StreamLayout<Real>::hps(L);
   const uint32_t bytes = static_cast<uint32_t>(hps * sizeof(Real));
   // [9 mbarriers][9 load counters] in 128 bytes, then the 9 half-plane buffers
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(slice + slice_spin_offset(tp, sy.ring));
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(slice + slice_spin_offset(tp, sy.ring, kMeterBytes<Real>));
   uint32_t* issued = reinterpret_cast<uint32_t*>(mbar + kSlots);
-  Real* buf = reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring) + 128);
+  Real* buf = reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring, kMeterBytes<Real>) + 128);
   // a resumable run keeps the path's lattice in its state; otherwise the
   // group's own HBM buffer holds it for the run
   unsigned char* st = path_state(P, sys_idx, path);
@@ -1749,7 +1793,7 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   const Real J = static_cast<Real>(sy.J), hf = static_cast<Real>(sy.h);
   const Couplings<Real> cp(P.systems + sys_idx);
   const int64_t j_first = P.s_begin > P.n_therm ? P.s_begin - P.n_therm : 0;
-  Meter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
+  PathMeter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
                     reinterpret_cast<Real*>(slice + slice_red_offset()),
                     sy.ring, tp >> 5, tid & 31, tid >> 5, tid,
                     1.0 / static_cast<double>(sy.N), J, hf, j_first};
