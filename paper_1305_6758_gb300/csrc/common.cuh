@@ -22,8 +22,8 @@ __host__ __device__ inline int path_init_mode(int32_t mode, int64_t path, int64_
 
 constexpr int kAccDoubles = 24;      // FP64 per-path accumulators (>= MP_NREC) in shared memory
 constexpr int kRedSlots = 4;         // partial sums per warp in the per-sweep reduction
-// Their bytes in shared memory: numbers of up to 8 bytes, or (FP64 form)
-// 96-bit integers.
+// Their bytes in shared memory: numbers of up to 8 bytes, or (FP64 simple cubic
+// lattices in shared memory) 96-bit integers.
 constexpr int kRedBytes = kRedSlots * 8, kRedBytesFix = kRedSlots * 12;
 constexpr int kMaxCta = 1024;
 // Most paths one CTA can hold: one warp each (groups of more than one warp

@@ -108,11 +108,6 @@ void ising_thresholds(const mp_system& s, unsigned long long* t) {
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
-// Bytes of a path's partial sums per warp and measurement sweep.
-int meter_bytes(const mp_system& s, int precision) {
-  return precision == MP_FP64 && s.lattice != MP_LATTICE_ISING ? kRedBytesFix : kRedBytes;
-}
-
 // Streamed lattices: one half-plane (one colour of one z-plane, 3 L^2/2 values)
 // padded to 16 bytes, in bytes.
 int half_plane_bytes(int L, int real) { return round_up(3 * (L * L / 2) * real, 16); }
@@ -131,6 +126,11 @@ bool streamed(const mp_system& s, int precision, uint32_t flags) {
          ((flags & MP_FLAG_STREAM) || !sweep_supports_L(precision, s.L));
 }
 
+// Bytes of a path's partial sums per warp and measurement sweep.
+int meter_bytes(const mp_system& s, int precision, uint32_t flags) {
+  return precision == MP_FP64 && s.lattice == MP_LATTICE_SC && !streamed(s, precision, flags) ? kRedBytesFix : kRedBytes;
+}
+
 // Lattices to stream whose ring of nine half-planes does not fit one SM's
 // shared memory (FP64 L >= 46, FP32 L >= 66; `optin` is the device's largest
 // shared memory per CTA, of which the kernels' static data take under 4 KB)
@@ -139,7 +139,7 @@ bool streamed(const mp_system& s, int precision, uint32_t flags) {
 bool in_place(const mp_system& s, int precision, uint32_t flags, int optin) {
   if (!streamed(s, precision, flags)) return false;
   const int real = precision == MP_FP64 ? 8 : 4;
-  return 128 + 9 * half_plane_bytes(s.L, real) + slice_spin_offset(32, 1, meter_bytes(s, precision)) > optin - 4096;
+  return 128 + 9 * half_plane_bytes(s.L, real) + slice_spin_offset(32, 1, kRedBytes) > optin - 4096;
 }
 
 }  // namespace
@@ -511,7 +511,7 @@ int plan(mp_state* h, const mp_config* cfg) {
   for (int k = 0; k < n; ++k) {
     const int64_t N = sites_of(h->systems[k]);
     const int NH = static_cast<int>((N + 1) / 2);
-    const int red = meter_bytes(h->systems[k], h->precision);
+    const int red = meter_bytes(h->systems[k], h->precision, h->flags);
     int t = (static_cast<int>(h->tp_override.size()) > k && h->tp_override[k] > 0) ? h->tp_override[k]
                                                                                   : cfg->threads_per_path;
     const bool by_default = t == 0;

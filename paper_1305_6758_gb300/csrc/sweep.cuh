@@ -878,10 +878,11 @@ __device__ __forceinline__ void sum_sites(const Geom& geo, const float* sp, int 
 // R sweeps is flushed into the FP64 accumulators by all warps together after
 // the next barrier while the other half fills, so no warp carries the
 // bookkeeping alone and no FP64 operation runs per sweep.
-// kFix (FP64 form): the partial sums are 96-bit integers, added up exactly over
-// the warps and rounded once, so that a path's record does not depend on how
-// many threads ran it: the planner chooses them by the paths per SM, and
-// processes that each run a part of an ensemble reproduce one that runs all.
+// kFix (FP64 simple cubic lattices in shared memory): the partial sums are
+// 96-bit integers, added up exactly over the warps and rounded once, so that a
+// path's record does not depend on how many threads ran it: the planner chooses
+// them by the paths per SM, and processes that each run a part of an ensemble
+// reproduce one that runs all.  Elsewhere the number depends on the lattice alone.
 template <typename Real, bool kFix = false>
 struct Meter {
   double* acc;
@@ -951,15 +952,20 @@ struct Meter {
   }
   // Store this warp's partials of the current measurement sweep and move to
   // the next (every lane calls, once per measurement sweep, in order).
-  // FP64 form: exact integers, three words each.
+  // FP64 form: the warp's sums are exact integers; lane k < 4 has sum k.
   __device__ void record(Partials<double> part) {
     // lanes 0 .. 3: E, M_y, M_x, M_z
     const Wide v = warp_sums(part.eb, part.mx, part.my, part.mz, lane);
     if (lane < 4) {
-      uint32_t* r = words(cur, slot_off + warp) + 3 * (lane == 1 ? 2 : lane == 2 ? 1 : lane);
-      r[0] = v.w0;
-      r[1] = v.w1;
-      r[2] = v.w2;
+      const int k = lane == 1 ? 2 : lane == 2 ? 1 : lane;
+      if constexpr (kFix) {
+        uint32_t* r = words(cur, slot_off + warp) + 3 * k;
+        r[0] = v.w0;
+        r[1] = v.w1;
+        r[2] = v.w2;
+      } else {
+        (cur_slot() + (slot_off + warp) * kRedSlots)[k] = v.real(lane == 0 ? kEnergyBits : kFixBits);
+      }
     }
     advance();
   }
@@ -1067,12 +1073,17 @@ struct Meter {
       if (lane == 0) acc[k] += static_cast<double>(v);
     }
   }
+  static __device__ __noinline__ void flush_call(Meter m, int64_t j0, int n) { m.flush(j0, n); }
   // At measurement sweep j (the current one), after its first barrier: flush
-  // the previous half.
+  // the previous half.  kCall: as a call, which leaves the sweep loop the
+  // registers that the integer sums would take: FP64 L = 16, 3072 paths, 200 sweeps:
+  // 39.1 -> 38.5 ms, L = 12 and 20 1.7% (not the one-site form: 1.21 -> 1.26 ms).
+  template <bool kCall = false>
   __device__ void maybe_flush(int64_t j) const {
     if ((cur == 0 || cur == R) && j > j_first) {
       const int64_t j0 = j - R > j_first ? j - R : j_first;
-      flush(j0, static_cast<int>(j - j0));
+      if constexpr (kCall) flush_call(*this, j0, static_cast<int>(j - j0));
+      else flush(j0, static_cast<int>(j - j0));
     }
   }
   // After the call's last sweep and its barrier: flush the rest of the
@@ -1127,11 +1138,10 @@ struct Meter {
   }
 };
 
-// The measurement state of the Heisenberg kernels and its bytes per warp and sweep.
-template <typename Real>
-using PathMeter = Meter<Real, sizeof(Real) == 8>;
-template <typename Real>
-constexpr int kMeterBytes = sizeof(Real) == 8 ? kRedBytesFix : kRedBytes;
+// The measurement state of a path in a geometry: exact sums where the number of
+// threads may go by the load; those sweeps also call the flush.
+template <typename Real, class Geom>
+constexpr bool kExactSums = sizeof(Real) == 8 && Geom::kColumns;
 
 // Initial spin of site i: uniform on the sphere (Sec. 2.2), uniform angles,
 // or the ordered start of Sec. 5.
@@ -1205,7 +1215,8 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
                                          int tid, int tp, int bar, Real* hbm_spins = nullptr) {
   using A = Arith<Real>;
   static_assert(!kWide || (sizeof(Real) == 4 && Geom::kColumns && !kOne), "wide paths are FP32 column walks");
-  Real* sp = hbm_spins ? hbm_spins : reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring, kMeterBytes<Real>));
+  constexpr bool kExact = kExactSums<Real, Geom>;
+  Real* sp = hbm_spins ? hbm_spins : reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring, kExact ? kRedBytesFix : kRedBytes));
   const int S = geo.stride();
   const uint32_t c2 = static_cast<uint32_t>(sy.path_begin + path);  // path id
   const uint32_t c3u = kTagUpdate | (static_cast<uint32_t>(sys_idx) << 8);
@@ -1231,7 +1242,7 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
     }
   }
   const int64_t j_first = P.s_begin > P.n_therm ? P.s_begin - P.n_therm : 0;
-  PathMeter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
+  Meter<Real, kExact> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
                     reinterpret_cast<Real*>(slice + slice_red_offset()),
                     sy.ring, (kWide ? sy.tm : tp) >> 5, tid & 31, tid >> 5, tid,
                     1.0 / static_cast<double>(sy.N), J, hf, j_first};
@@ -1350,7 +1361,7 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
         canceled = true;
         break;
       }
-      meter.maybe_flush(j);
+      meter.template maybe_flush<kExact>(j);
       half_sweep<Real, Geom, true, true>(geo, 1, pre, P.key, sp, tid, tp, K, units, cp, accepted, part);
       meter.record(part);
       group_sync(tp, bar);
@@ -1512,7 +1523,7 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
   constexpr int HL = G::HL, HP = G::HP, ZL = G::ZL, S = G::S;
   constexpr int NH = L * L * L / 2;  // sites per colour of the whole lattice
   // rank 0's ring holds the partials of both CTAs' warps
-  Real* sp = reinterpret_cast<Real*>(slice + slice_spin_offset(2 * tp, sy.ring, kMeterBytes<Real>));
+  Real* sp = reinterpret_cast<Real*>(slice + slice_spin_offset(2 * tp, sy.ring, kRedBytes));
   Real* partner_sp = map_rank(sp, rank ^ 1u);
   const int zbase = static_cast<int>(rank) * ZL;
   const uint32_t c2 = static_cast<uint32_t>(sy.path_begin + path);  // path id
@@ -1523,7 +1534,7 @@ __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, co
   const Couplings<Real> cp(P.systems + sys_idx);
   const int64_t j_first = P.s_begin > P.n_therm ? P.s_begin - P.n_therm : 0;
   Real* red0 = reinterpret_cast<Real*>(slice + slice_red_offset());
-  PathMeter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
+  Meter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
                     rank == 0 ? red0 : map_rank(red0, 0u),
                     sy.ring, tp >> 5, tid & 31, tid >> 5, tid,
                     1.0 / static_cast<double>(sy.N), J, hf, j_first};
@@ -1777,9 +1788,9 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   const int hps = StreamLayout<Real>::hps(L);
   const uint32_t bytes = static_cast<uint32_t>(hps * sizeof(Real));
   // [9 mbarriers][9 load counters] in 128 bytes, then the 9 half-plane buffers
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(slice + slice_spin_offset(tp, sy.ring, kMeterBytes<Real>));
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(slice + slice_spin_offset(tp, sy.ring, kRedBytes));
   uint32_t* issued = reinterpret_cast<uint32_t*>(mbar + kSlots);
-  Real* buf = reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring, kMeterBytes<Real>) + 128);
+  Real* buf = reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring, kRedBytes) + 128);
   // a resumable run keeps the path's lattice in its state; otherwise the
   // group's own HBM buffer holds it for the run
   unsigned char* st = path_state(P, sys_idx, path);
@@ -1793,7 +1804,7 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   const Real J = static_cast<Real>(sy.J), hf = static_cast<Real>(sy.h);
   const Couplings<Real> cp(P.systems + sys_idx);
   const int64_t j_first = P.s_begin > P.n_therm ? P.s_begin - P.n_therm : 0;
-  PathMeter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
+  Meter<Real> meter{reinterpret_cast<double*>(slice + slice_acc_offset()),
                     reinterpret_cast<Real*>(slice + slice_red_offset()),
                     sy.ring, tp >> 5, tid & 31, tid >> 5, tid,
                     1.0 / static_cast<double>(sy.N), J, hf, j_first};
