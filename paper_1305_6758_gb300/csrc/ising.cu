@@ -44,6 +44,12 @@ namespace {
 
 constexpr int kIsingThreads = 1024;
 constexpr uint32_t kOnes = 0x01010101u;
+// A thread counts its accepted flips in 32 bits; every kAcceptFold sweeps the
+// warp's sum, still below 2^32, goes to the path's total in FP64 (exact to 2^53).
+// (In a loop of its own: a 64-bit count per thread, or a test in the sweep loop,
+// costs registers that the kernel does not have, L = 60 0.5%, L = 6 1.2%.)
+constexpr uint32_t kAcceptFold = 1u << 15;
+static_assert(uint64_t{kAcceptFold} * MP_ISING_MAX_L * MP_ISING_MAX_L < uint64_t{1} << 32, "all flips of a lattice");
 
 // Blocks per segment for tp threads: the walk takes rounds x (q + what a
 // segment's start costs, about 0.4 of a strip).
@@ -81,7 +87,8 @@ struct StripWalk {
 };
 
 struct IsingSums {
-  int accepted, up_own, up_nb, up_pairs;
+  uint32_t accepted;
+  int up_own, up_nb, up_pairs;
 };
 
 // Flip tests of colour kC for this thread's strips.  table: shared-memory
@@ -153,7 +160,7 @@ __device__ __forceinline__ void ising_half_sweep(const StripWalk& w, const Philo
     for (; left > 0; --left) strip(std::false_type{});
     if (short_end) strip(std::true_type{});
     if (g == 0) own[hx + w.S] = own[hx];  // read as row L's block in the next half-sweep
-    sum.accepted = __dp4a(flips, kOnes, static_cast<uint32_t>(sum.accepted));
+    sum.accepted = __dp4a(flips, kOnes, sum.accepted);
     if (kMeas) sum.up_own = __dp4a(ups, kOnes, static_cast<uint32_t>(sum.up_own));
     g += w.dg;
     hx += w.dh;
@@ -215,7 +222,8 @@ __device__ void run_path_ising(const DevSystem& sy, int sys_idx, int64_t path,
     sp[t] = word;
   }
   if (tid < kAccDoubles) meter.acc[tid] = resume ? reinterpret_cast<const double*>(st)[tid] : 0.0;
-  const double accepted_before = resume ? reinterpret_cast<const double*>(st)[kAccDoubles] : 0.0;
+  double accepted_before = resume ? reinterpret_cast<const double*>(st)[kAccDoubles] : 0.0;
+  double* const accepted = meter.acc + MP_R_ACC;  // accepted flips of this call; the meter leaves the place alone
   if (tid == 0) cancel_flag[gidx] = 0;
   group_sync(tp, bar);
 
@@ -235,44 +243,53 @@ __device__ void run_path_ising(const DevSystem& sy, int sys_idx, int64_t path,
   const int g0 = tid / HL, h0 = tid - g0 * HL;
   auto sweep = [&](auto wide_c) {
     constexpr bool kWide = decltype(wide_c)::value;
-    for (int64_t s = P.s_begin; s < P.s_end; ++s) {
-      const uint32_t sw = static_cast<uint32_t>(s);
-      const PhiloxPrefix pa = philox_prefix(sw, c2, c3a, P.key), pb = philox_prefix(sw, c2, c3b, P.key);
-      sum.up_own = sum.up_nb = sum.up_pairs = 0;
-      poll_cancel(P, s, tid, &cancel_flag[gidx]);
-      const bool meas = s >= P.n_therm;
-      if (meas)
-        ising_half_sweep<0, kWide, true, false>(walk, pa, P.key, sp0, sp1, table, tid, tp, h0, g0, sum);
-      else
-        ising_half_sweep<0, kWide, false, false>(walk, pa, P.key, sp0, sp1, table, tid, tp, h0, g0, sum);
-      group_sync(tp, bar);
-      if (cancel_flag[gidx]) {
-        canceled = true;
-        break;
-      }
-      if (!meas) {
-        ising_half_sweep<1, kWide, false, false>(walk, pb, P.key, sp1, sp0, table, tid, tp, h0, g0, sum);
+    for (int64_t s = P.s_begin; s < P.s_end && !canceled;) {
+      const uint32_t last = static_cast<uint32_t>(min(s | static_cast<int64_t>(kAcceptFold - 1), P.s_end - 1));
+      for (;; ++s) {
+        const uint32_t sw = static_cast<uint32_t>(s);
+        const PhiloxPrefix pa = philox_prefix(sw, c2, c3a, P.key), pb = philox_prefix(sw, c2, c3b, P.key);
+        sum.up_own = sum.up_nb = sum.up_pairs = 0;
+        poll_cancel(P, s, tid, &cancel_flag[gidx]);
+        const bool meas = s >= P.n_therm;
+        if (meas)
+          ising_half_sweep<0, kWide, true, false>(walk, pa, P.key, sp0, sp1, table, tid, tp, h0, g0, sum);
+        else
+          ising_half_sweep<0, kWide, false, false>(walk, pa, P.key, sp0, sp1, table, tid, tp, h0, g0, sum);
         group_sync(tp, bar);
-        continue;
+        if (cancel_flag[gidx]) {
+          canceled = true;
+          break;
+        }
+        if (!meas) {
+          ising_half_sweep<1, kWide, false, false>(walk, pb, P.key, sp1, sp0, table, tid, tp, h0, g0, sum);
+          group_sync(tp, bar);
+          if (sw == last) break;
+          continue;
+        }
+        const int64_t j = s - P.n_therm;
+        meter.maybe_flush(j);
+        const int ups0 = sum.up_own;
+        ising_half_sweep<1, kWide, true, true>(walk, pb, P.key, sp1, sp0, table, tid, tp, h0, g0, sum);
+        // exact integers, then one slot of the ring: over the warp's sites
+        // sum s = 2 (spins up) - sites, and over its colour-1 sites, with s = 2 b - 1
+        // and neighbour sum 2 n - 4, sum s (2 n - 4) = 4 sum b n - 8 sum b - 2 sum n + 4 sites
+        const int b1 = __reduce_add_sync(0xffffffffu, sum.up_own - ups0), b0 = __reduce_add_sync(0xffffffffu, ups0);
+        const int nn = __reduce_add_sync(0xffffffffu, sum.up_nb), bn = __reduce_add_sync(0xffffffffu, sum.up_pairs);
+        if ((tid & 31) == 0) {
+          double* r = meter.cur_slot() + (tid >> 5) * kRedSlots;
+          r[0] = static_cast<double>(4 * bn - 8 * b1 - 2 * nn + 4 * warp_sites);
+          r[1] = 0.0;
+          r[2] = 0.0;
+          r[3] = static_cast<double>(2 * (b0 + b1) - 2 * warp_sites);
+        }
+        meter.advance();
+        group_sync(tp, bar);
+        if (sw == last) break;
       }
-      const int64_t j = s - P.n_therm;
-      meter.maybe_flush(j);
-      const int ups0 = sum.up_own;
-      ising_half_sweep<1, kWide, true, true>(walk, pb, P.key, sp1, sp0, table, tid, tp, h0, g0, sum);
-      // exact integers, then one slot of the ring: over the warp's sites
-      // sum s = 2 (spins up) - sites, and over its colour-1 sites, with s = 2 b - 1
-      // and neighbour sum 2 n - 4, sum s (2 n - 4) = 4 sum b n - 8 sum b - 2 sum n + 4 sites
-      const int b1 = __reduce_add_sync(0xffffffffu, sum.up_own - ups0), b0 = __reduce_add_sync(0xffffffffu, ups0);
-      const int nn = __reduce_add_sync(0xffffffffu, sum.up_nb), bn = __reduce_add_sync(0xffffffffu, sum.up_pairs);
-      if ((tid & 31) == 0) {
-        double* r = meter.cur_slot() + (tid >> 5) * kRedSlots;
-        r[0] = static_cast<double>(4 * bn - 8 * b1 - 2 * nn + 4 * warp_sites);
-        r[1] = 0.0;
-        r[2] = 0.0;
-        r[3] = static_cast<double>(2 * (b0 + b1) - 2 * warp_sites);
-      }
-      meter.advance();
-      group_sync(tp, bar);
+      ++s;
+      const uint32_t flips = __reduce_add_sync(0xffffffffu, sum.accepted);
+      if ((tid & 31) == 0) atomicAdd(accepted, static_cast<double>(flips));
+      sum.accepted = 0;
     }
   };
   if (wide) sweep(std::true_type{});
@@ -288,6 +305,11 @@ __device__ void run_path_ising(const DevSystem& sy, int sys_idx, int64_t path,
   const int64_t n_meas_done = P.s_end > P.n_therm ? P.s_end - P.n_therm : 0;
   meter.finish(n_meas_done);
   group_sync(tp, bar);
+  if (tid == 0) {
+    accepted_before += *accepted;
+    *accepted = 0.0;
+  }
+  __syncwarp();  // the first warp saves the accumulators
   if (P.save && st) {
     for (int i = tid; i < N; i += tp) {
       const int x = i % L, y = i / L;
@@ -295,7 +317,7 @@ __device__ void run_path_ising(const DevSystem& sy, int sys_idx, int64_t path,
     }
     if (tid < kAccDoubles) reinterpret_cast<double*>(st)[tid] = meter.acc[tid];
   }
-  meter.write_record(P.records + (sy.rec_offset + path) * MP_NREC, sum.accepted, 0.0, P.s_end,
+  meter.write_record(P.records + (sy.rec_offset + path) * MP_NREC, 0, 0.0, P.s_end,
                      n_meas_done, N, tp, bar, accepted_before,
                      (P.save && st) ? reinterpret_cast<double*>(st) + kAccDoubles : nullptr);
   if (P.spins != nullptr) {
