@@ -136,6 +136,17 @@ struct Attempt<double> {
   }
 };
 
+// f / N correctly rounded, for f an FP32 number and invN = 1 / N correctly
+// rounded: the product's residual is exact and corrects it (P. Markstein, IBM J.
+// Res. Dev. 34, 1990); f / N keeps 2^-31 of an ulp from every midpoint of two
+// doubles (f has 24 bits and N fewer than 31), far more than what is neglected.
+// Three FP64 instructions of 76 cycles each instead of a division's ten.
+__device__ __forceinline__ double per_site(double f, double dN, double invN) {
+  const double q = __dmul_rn(f, invN);
+  if ((__double2hiint(q) & 0x7ff00000) == 0x7ff00000) return q;  // infinity, NaN
+  return __fma_rn(__fma_rn(-q, dN, f), invN, q);
+}
+
 // Sums of one measurement: bonds and spins over all sites.  FP32: added one
 // by one in site order (lane 0 the bonds, lanes 1 to 3 a component each, from
 // the dot products that the 32 lanes leave in `dots`), so that the sums are
@@ -230,7 +241,7 @@ __device__ void run_path_random(const DevSystem* sy, int sys_idx, int64_t path, 
   double acc = 0.0;  // lane k: record field k
   int64_t accepted = 0;
   const uint32_t before = (1u << lane) - 1u;
-  const double dN = static_cast<double>(N), invN = 1.0 / dN;
+  const double dN = static_cast<double>(N), invN = __drcp_rn(dN);
   const int64_t S_total = P.n_therm + P.n_meas;
   for (int64_t s = 0; s < S_total; ++s) {
     const PhiloxPrefix pre = philox_prefix(static_cast<uint32_t>(s), c2, kTagSite | sys_hi, P.key);
@@ -283,8 +294,7 @@ __device__ void run_path_random(const DevSystem* sy, int sys_idx, int64_t path, 
       const float en = -cp.J * part.eb - cp.hf * part.mz;
       v = static_cast<double>(lane == 0 ? en : lane == 1 ? part.mx : lane == 2 ? part.my : part.mz);
     }
-    // (FP32 sums: a multiplication, one FP64 instruction instead of ten)
-    v = sizeof(Real) == 8 ? __ddiv_rn(v, dN) : __dmul_rn(v, invN);
+    v = sizeof(Real) == 8 ? __ddiv_rn(v, dN) : per_site(v, dN, invN);
     const double e = __shfl_sync(0xffffffffu, v, 0), mx = __shfl_sync(0xffffffffu, v, 1),
                  my = __shfl_sync(0xffffffffu, v, 2), mz = __shfl_sync(0xffffffffu, v, 3);
     const double m = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(mx, mx), __dmul_rn(my, my)), __dmul_rn(mz, mz)));
@@ -434,7 +444,7 @@ __device__ void run_path_thread(const DevSystem* sy, int sys_idx, int64_t path, 
   const int init = path_init_mode(P.init_mode, path, sy->n_paths);
   for (int i = 0; i < N; ++i) S.st(i, initial_spin<Real>(static_cast<uint32_t>(i), c2, kTagInit | sys_hi, P, init));
   const Couplings<Real> cp(sy);
-  const double dN = static_cast<double>(N);
+  const double dN = static_cast<double>(N), invN = __drcp_rn(dN);
   double acc[MP_R_ACC];
 #pragma unroll
   for (int q = 0; q < MP_R_ACC; ++q) acc[q] = 0.0;
@@ -489,11 +499,10 @@ __device__ void run_path_thread(const DevSystem* sy, int sys_idx, int64_t path, 
       my = __ddiv_rn(part.my.real() * kSpinUnit, dN);
       mz = __ddiv_rn(mz, dN);
     } else {
-      const double invN = 1.0 / dN;
-      e = static_cast<double>(-cp.J * part.eb - cp.hf * part.mz) * invN;
-      mx = static_cast<double>(part.mx) * invN;
-      my = static_cast<double>(part.my) * invN;
-      mz = static_cast<double>(part.mz) * invN;
+      e = per_site(static_cast<double>(-cp.J * part.eb - cp.hf * part.mz), dN, invN);
+      mx = per_site(static_cast<double>(part.mx), dN, invN);
+      my = per_site(static_cast<double>(part.my), dN, invN);
+      mz = per_site(static_cast<double>(part.mz), dN, invN);
     }
     const double m = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(mx, mx), __dmul_rn(my, my)), __dmul_rn(mz, mz)));
     const double now[MP_R_ACC] = {e, __dmul_rn(e, e), m, __dmul_rn(m, m), __dmul_rn(__dmul_rn(__dmul_rn(m, m), m), m),
