@@ -356,11 +356,11 @@ __global__ void __launch_bounds__(kIsingThreads, 1) ising_kernel(const SweepPara
 // 32; 13 reach 0.56, 26 0.94 of the rate, at L = 128) and with the barrier that
 // more than one warp per path needs (about 7%).  Attempts/s by threads per path:
 // L = 60 32: 1.02e12, 64: 9.3e11, 256: 6.5e11; L = 100 32: 7.9e11, 64: 9.3e11.
-int ising_threads(int L, int64_t paths_per_sm, int smem_max, int ring) {
+int ising_threads(int L, int64_t paths_per_sm, int smem_max, int ring, int most) {
   const int S = (L / 2) * ((L + 3) / 4);
   double best = -1.0;
   int best_t = 32;
-  for (int t = 32; t <= kIsingThreads && (t == 32 || t < 2 * S); t += 32) {
+  for (int t = 32; t <= most && (t == 32 || t < 2 * S); t += 32) {
     const int slice = (slice_spin_offset(t, ring, kRedBytes) + ising_slice_spin_bytes(L) + 127) / 128 * 128;
     int64_t fit = std::min<int64_t>(smem_max / slice, t > 32 ? std::min(15, kIsingThreads / t) : kIsingThreads / t);
     fit = std::min(fit, paths_per_sm);

@@ -454,6 +454,9 @@ int plan(mp_state* h, const mp_config* cfg) {
     r = best_r;
     sl = best_sl;
   };
+  // most threads per path that a default may take: those of the CTA, where the
+  // caller gives its size
+  const int tp_max = cfg->cta_threads > 0 ? std::min(cta_max, cfg->cta_threads) : cta_max;
   int max_tp = 32;
   int64_t batch_paths = 0;
   for (const mp_system& sy : h->systems) batch_paths += sy.n_paths;
@@ -479,7 +482,7 @@ int plan(mp_state* h, const mp_config* cfg) {
     const double n_meas = static_cast<double>(h->n_meas), n_all = static_cast<double>(h->n_therm) + n_meas;
     const int64_t load = (batch_paths + sms - 1) / sms;  // paths per SM
     double best = 0.0;
-    for (int c = tp[k]; c <= std::min(cta_max, round_up(NH, 32)); c += 32) {
+    for (int c = tp[k]; c <= std::min(tp_max, round_up(NH, 32)); c += 32) {
       const int s = round_up(slice_spin_offset(c, ring[k], kRedBytes) + static_cast<int>(lat), 128);
       int64_t fit = std::min<int64_t>(smem_max / s, c > 32 ? std::min(15, cta_max / c) : cta_max / c);
       fit = std::min(fit, load);
@@ -571,18 +574,20 @@ int plan(mp_state* h, const mp_config* cfg) {
     // depend on the number of threads, which is chosen by the paths that an SM
     // gets; it does depend on the ring (the sweeps summed together), which is
     // therefore that of the threads chosen for a full GPU.
-    std::function<int(int64_t, int)> by_load;  // threads for so many paths per SM and this ring
+    std::function<int(int64_t, int, int)> by_load;  // threads for so many paths per SM, this ring, at most so many
     if (h->systems[k].lattice == MP_LATTICE_ISING) {
-      by_load = [&](int64_t per_sm, int r) { return ising_threads(h->systems[k].L, per_sm, smem_max, r); };
+      by_load = [&](int64_t per_sm, int r, int most) {
+        return ising_threads(h->systems[k].L, per_sm, smem_max, r, most);
+      };
     } else if (h->systems[k].lattice == MP_LATTICE_SC && real == 8) {
       // FP64 lattices are large (L = 16: two paths per SM): the count that fills
       // its own lanes best, weighed with the warps the SM then holds (of 16).  L =
       // 16, 3072 paths: 6.2e10 attempts/s with 128 threads, 7.3e10 with 256; L = 20,
       // 500 paths: 3.4e10 with 160, 6.2e10 with 512.
-      by_load = [&](int64_t per_sm, int r) {
+      by_load = [&](int64_t per_sm, int r, int most) {
         double best = -1.0;
         int best_t = 0;
-        for (int c = 32; c <= std::min(cta_max, round_up(NH, 32)); c += 32) {
+        for (int c = 32; c <= std::min(most, round_up(NH, 32)); c += 32) {
           const int units = h->systems[k].L * h->systems[k].L / 2 * column_segments(h->systems[k].L, 1, c);
           int64_t fit = std::min<int64_t>(smem_max / need_of(c, r), c > 32 ? std::min(15, cta_max / c) : cta_max / c);
           fit = std::min(fit, per_sm);
@@ -597,7 +602,7 @@ int plan(mp_state* h, const mp_config* cfg) {
         return best_t;
       };
     }
-    if (t == 0 && by_load) t = by_load(INT64_MAX, h->systems[k].lattice == MP_LATTICE_ISING ? 16 : 1);
+    if (t == 0 && by_load) t = by_load(INT64_MAX, h->systems[k].lattice == MP_LATTICE_ISING ? 16 : 1, cta_max);
     if (t == 0 && h->systems[k].lattice == MP_LATTICE_SC) {
       // a divisor of the sites per colour lets each thread walk a block of
       // columns; pick the one closest to the target sites per thread
@@ -618,7 +623,7 @@ int plan(mp_state* h, const mp_config* cfg) {
     ring[k] = 16;
     pick_ring(ring[k], slice[k], [&]() { return need_of(t, ring[k]); }, t);
     if (by_default && by_load) {
-      const int loaded = by_load((batch_paths + sms - 1) / sms, ring[k]);
+      const int loaded = by_load((batch_paths + sms - 1) / sms, ring[k], tp_max);
       if (loaded > 0) {
         t = loaded;
         slice[k] = need_of(t, ring[k]);
