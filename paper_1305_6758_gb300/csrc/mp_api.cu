@@ -5,6 +5,7 @@
 // queue, the device buffers (per-path records, estimates, optional final
 // spins) and, with MP_FLAG_GRAPH, a CUDA graph of one run: zero the queue,
 // the sweep kernel, the reduction kernel, with timing events between them.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -196,7 +197,8 @@ struct mp_state {
   int64_t sweeps_done = 0;         // progress of the resumable schedule
   int* h_cancel = nullptr;         // host-mapped cancel flag
   int* d_cancel = nullptr;
-  int cancel_slot = -1;            // its slot in the process's pool, -1: an allocation of its own
+  int cancel_slot = -1;            // its slot in the device's pool, -1: an allocation of its own
+  int cancel_generation = 0;       // of the pool's block
   int64_t lattice_stride = 0;      // bytes per (CTA, group) lattice buffer
   int lattice_groups = 0;          // buffers per CTA
   std::vector<void*> owned;
@@ -277,29 +279,60 @@ void dev_free(mp_state* h, void* p) {
 }
 
 // The handles' cancel flags: host memory the kernels can read while they run.
-// Pinned allocations cost 0.1 ms each way, so flags come from one block of
-// kCancelSlots cache lines per process, and return to it; handles beyond that
-// allocate their own.
+// Pinned allocations cost 0.1 ms each way, so the flags of a device's handles come
+// from one block of kCancelSlots cache lines, and return to it; handles beyond
+// that allocate their own.  The block lives as long as the device's context: a
+// cudaDeviceReset takes it away, and its address may then be anyone's, so it is
+// known by the id that the driver gives every allocation.
 constexpr int kCancelSlots = 256, kCancelStride = 64 / static_cast<int>(sizeof(int));
+constexpr int kCancelDevices = 64;
+struct CancelPool {
+  int* base = nullptr;
+  unsigned long long id = 0;  // of the allocation at base
+  int generation = 0;         // blocks so far
+  std::vector<int> free;
+};
 std::mutex g_cancel_mu;
-int* g_cancel_base = nullptr;
-std::vector<int> g_cancel_free;
+CancelPool g_cancel[kCancelDevices];
+
+// The driver's id of the allocation at p, unique in the process; 0: none there.
+unsigned long long allocation_id(const void* p) {
+  using Get = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+  static const Get get = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &r);
+    return e == cudaSuccess && r == cudaDriverEntryPointSuccess ? reinterpret_cast<Get>(f) : nullptr;
+  }();
+  unsigned long long id = 0;
+  if (!get || get(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return 0;
+  return id;
+}
 
 cudaError_t cancel_acquire(mp_state* h) {
-  {
+  if (h->device < kCancelDevices) {
     std::lock_guard<std::mutex> lock(g_cancel_mu);
-    if (!g_cancel_base) {
+    CancelPool& pool = g_cancel[h->device];
+    if (pool.base && allocation_id(pool.base) != pool.id) pool.base = nullptr;  // gone with its context
+    if (!pool.base) {
       void* p = nullptr;
-      const cudaError_t e = cudaHostAlloc(&p, kCancelSlots * kCancelStride * sizeof(int),
-                                          cudaHostAllocMapped | cudaHostAllocPortable);
+      const cudaError_t e = cudaHostAlloc(&p, kCancelSlots * kCancelStride * sizeof(int), cudaHostAllocMapped);
       if (e != cudaSuccess) return e;
-      g_cancel_base = static_cast<int*>(p);
-      for (int k = kCancelSlots - 1; k >= 0; --k) g_cancel_free.push_back(k);
+      pool.id = allocation_id(p);
+      if (pool.id == 0) {
+        cudaFreeHost(p);  // no telling it apart later: no pool
+      } else {
+        pool.base = static_cast<int*>(p);
+        ++pool.generation;
+        pool.free.clear();
+        for (int k = kCancelSlots - 1; k >= 0; --k) pool.free.push_back(k);
+      }
     }
-    if (!g_cancel_free.empty()) {
-      h->cancel_slot = g_cancel_free.back();
-      g_cancel_free.pop_back();
-      h->h_cancel = g_cancel_base + h->cancel_slot * kCancelStride;
+    if (pool.base && !pool.free.empty()) {
+      h->cancel_slot = pool.free.back();
+      pool.free.pop_back();
+      h->cancel_generation = pool.generation;
+      h->h_cancel = pool.base + h->cancel_slot * kCancelStride;
     }
   }
   if (h->cancel_slot < 0) {
@@ -316,7 +349,8 @@ void cancel_release(mp_state* h) {  // after the handle's stream has drained
     cudaFreeHost(h->h_cancel);
   } else {
     std::lock_guard<std::mutex> lock(g_cancel_mu);
-    g_cancel_free.push_back(h->cancel_slot);
+    CancelPool& pool = g_cancel[h->device];
+    if (pool.generation == h->cancel_generation) pool.free.push_back(h->cancel_slot);
   }
   h->h_cancel = nullptr;
 }
