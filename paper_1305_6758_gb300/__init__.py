@@ -249,7 +249,7 @@ class Simulation:
         cfg.threads_per_path = threads_per_path
         self.n_therm, self.n_meas, self.precision = n_therm, n_meas, precision
         self._h = ctypes.c_void_p()
-        self._records = None  # view of the handle's record buffer (its address is fixed)
+        self._records = None  # over the handle's record buffer (its address is fixed); never handed out itself
         with torch.cuda.device(self.device):
             _check(lib.mp_create_ex(ctypes.byref(cfg), ctypes.byref(self._h)))
 
@@ -314,7 +314,7 @@ class Simulation:
             _check(_lib.mp_device_buffers(self._h, ctypes.byref(rec), None), self._h)
             total = sum(s.n_paths for s in self.systems)
             self._records = _wrap_device(rec.value, (total, NREC), self.device)
-        return self._records
+        return self._records.data  # a tensor of the caller's: shape, flags and version its own
 
     def backward(self, g_e, g_m):
         """Fluctuation-formula gradients (d/dbeta, d/dh) of g_e.<e> + g_m.<|m|> per system."""
