@@ -1240,10 +1240,16 @@ int mp_create_ex(const mp_config* cfg, mp_handle* out) {
     if (ce != cudaSuccess) return bail(cuda_fail(h, ce, "cancel flag"));
   }
   const int n = static_cast<int>(h->hsys.size());
-  // unit tables: at most L^3/2 units per simple cubic size that fits shared memory
+  // unit tables: for each simple cubic size that fits shared memory, whose
+  // systems share their layout, those of tp and of tm threads (and, while the
+  // autotuner tries a count on one of them, of that), at most L^3/2 units each
   h->units_capacity = 0;
-  for (const mp_system& s : h->systems)
-    if (s.lattice == MP_LATTICE_SC && s.L <= 26) h->units_capacity += static_cast<int64_t>(s.L) * s.L * s.L;
+  std::vector<char> seen(27, 0);
+  for (const mp_system& s : h->systems) {
+    if (s.lattice != MP_LATTICE_SC || s.L > 26 || seen[s.L]) continue;
+    seen[s.L] = 1;
+    h->units_capacity += static_cast<int64_t>(s.L) * s.L * s.L * 3 / 2;
+  }
   {  // one allocation: the tables (uploaded together), the queue, records, scratch, estimates and error word
     size_t size = 0;
     std::vector<std::pair<void**, size_t>> parts;
