@@ -69,7 +69,12 @@ extern "C" {
 #define MP_ISING_MAX_L 256
 
 #define MP_FP32 0 /* FP32 spins, dE and Boltzmann factor; FP64 accumulators */
-#define MP_FP64 1 /* FP64 throughout (the plain FP64 GPU form) */
+#define MP_FP64 1 /* the FP64 form: spin components as multiples of 2^-53 (64-bit
+                     integers; saved states and read-out spins are the doubles
+                     of the same value, and a restored state is rounded to
+                     them), every accept decision that of FP64 energy
+                     differences and Boltzmann factors of those spins, exact
+                     sums over the sites, FP64 accumulators */
 
 #define MP_INIT_SPHERE 0  /* uniform on the sphere (Sec. 4, "uniform state") */
 #define MP_INIT_ANGLES 1  /* theta, phi each uniform (Sec. 2.2 "both angles") */

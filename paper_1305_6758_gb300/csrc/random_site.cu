@@ -398,8 +398,7 @@ __global__ void __launch_bounds__(32 * kWarps) random_site_kernel(const SweepPar
 // 1.4e10 against 0.5e10; with 10^6 paths 1.6e11 against 2.7e10.  Lattices in HBM,
 // element (site i, path p) of system k at spin_offset[k] / 3 + i * P_k + p, so
 // that a warp's threads read consecutive elements of the same site.
-constexpr int kThreadSites = 16;
-constexpr int kThreadPaths = 4864;  // one warp per SM
+constexpr int kThreadSites = 16;  // and enough paths for a warp of them on every SM
 
 template <typename Real>
 struct ColumnStore;
@@ -568,7 +567,7 @@ cudaError_t random_site_plan(int precision, int64_t max_sites, int64_t total_pat
   cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   if (e != cudaSuccess) return e;
-  plan->thread_per_path = max_sites <= kThreadSites && total_paths >= kThreadPaths;
+  plan->thread_per_path = max_sites <= kThreadSites && total_paths >= int64_t{32} * sms;
   if (plan->thread_per_path) {
     plan->shared = false;
     plan->slice = plan->smem = 0;

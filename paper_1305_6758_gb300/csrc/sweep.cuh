@@ -69,7 +69,6 @@ struct Arith<float> {
     y = st * sp;
     z = ct;
   }
-  static __device__ __forceinline__ float add(float a, float b) { return a + b; }
   // a.b, every rounding spelled out: where a sum of products is left to the
   // compiler, which product it rounds first changes with the code around it,
   // and with it one accept decision in 1e8.
@@ -105,24 +104,15 @@ struct Arith<float> {
   }
 };
 
-// FP64 form: 32-bit uniforms (r + 1/2) 2^-32, IEEE sqrt, library sin/cos/exp,
-// and the local-field dot product rounded term by term in the order
-// ((dx hx + dy hy) + dz hz) with no fused multiply-add, so that dE matches a
-// plain FP64 evaluation bit for bit.
+// FP64 form: 32-bit uniforms (r + 1/2) 2^-32.  Trial spins are fix_trial's
+// (fixed64.cuh); where the FP32 stage does not decide a move, the local-field dot
+// product is rounded term by term in the order ((dx hx + dy hy) + dz hz) with no
+// fused multiply-add and the Boltzmann factor is the library's exp, so that dE is a
+// plain FP64 evaluation's of the same spins.
 template <>
 struct Arith<double> {
   static __device__ __forceinline__ double uni(uint32_t r) {
     return (static_cast<double>(r) + 0.5) * 0x1p-32;
-  }
-  static __device__ __forceinline__ void trial(uint32_t r0, uint32_t r1, double& x, double& y,
-                                               double& z) {
-    z = 2.0 * uni(r0) - 1.0;
-    const double rad = sqrt(__dmul_rn(1.0 - z, 1.0 + z));
-    const double phi = __dmul_rn(2.0 * 3.141592653589793, uni(r1));
-    double s, c;
-    sincos(phi, &s, &c);
-    x = __dmul_rn(rad, c);
-    y = __dmul_rn(rad, s);
   }
   static __device__ __forceinline__ void init_angles(uint32_t r0, uint32_t r1, double& x,
                                                      double& y, double& z) {
@@ -135,7 +125,6 @@ struct Arith<double> {
     y = __dmul_rn(st, sp);
     z = ct;
   }
-  static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
   static __device__ __forceinline__ double square(double x, double y, double z) {
     return fma(z, z, fma(y, y, x * x));
   }
@@ -150,7 +139,6 @@ struct Arith<double> {
     const double dE = delta_e(dx, dy, dz, hx, hy, hz, J, hf);
     return dE <= 0.0 || uni(r2) < exp(__dmul_rn(-beta, dE));
   }
-  static __device__ __forceinline__ double beta_param(double beta) { return beta; }
   static __device__ __forceinline__ double shfl(double v, int o) {
     return __shfl_xor_sync(0xffffffffu, v, o);
   }
@@ -1151,15 +1139,15 @@ __device__ __forceinline__ V3<Real> initial_spin(uint32_t i, uint32_t c2, uint32
   using S = Stored<Real>;
   const Philox4 r = philox4x32_10(i, 0u, c2, c3i, P.key);
   if (mode == MP_INIT_ORDERED) return V3<Real>{S::from(Real(0)), S::from(Real(0)), S::from(Real(1))};
-  if (mode == MP_INIT_SPHERE) {
-    if constexpr (sizeof(Real) == 8) {
-      const Fix3 t = fix_trial(r.x, r.y, fix_root(r.x), sine_shared());
-      return V3<Real>{t.x, t.y, t.z};
-    }
-  }
   Real x, y, z;
-  if (mode == MP_INIT_ANGLES) Arith<Real>::init_angles(r.x, r.y, x, y, z);
-  else Arith<Real>::trial(r.x, r.y, x, y, z);
+  if (mode == MP_INIT_ANGLES) {
+    Arith<Real>::init_angles(r.x, r.y, x, y, z);
+  } else if constexpr (sizeof(Real) == 8) {
+    const Fix3 t = fix_trial(r.x, r.y, fix_root(r.x), sine_shared());
+    return V3<Real>{t.x, t.y, t.z};
+  } else {
+    Arith<Real>::trial(r.x, r.y, x, y, z);
+  }
   return V3<Real>{S::from(x), S::from(y), S::from(z)};
 }
 
@@ -1213,7 +1201,6 @@ template <typename Real, class Geom, bool kOne = false, bool kWide = false>
 __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, int sys_idx,
                                          int64_t path, const SweepParams& P, unsigned char* slice,
                                          int tid, int tp, int bar, Real* hbm_spins = nullptr) {
-  using A = Arith<Real>;
   static_assert(!kWide || (sizeof(Real) == 4 && Geom::kColumns && !kOne), "wide paths are FP32 column walks");
   constexpr bool kExact = kExactSums<Real, Geom>;
   Real* sp = hbm_spins ? hbm_spins : reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring, kExact ? kRedBytesFix : kRedBytes));
@@ -1518,7 +1505,6 @@ __device__ __forceinline__ void half_sweep_pair(int c, int zbase, const PhiloxPr
 template <typename Real, int L>
 __device__ void run_path_pair(const DevSystem& sy, int sys_idx, int64_t path, const SweepParams& P,
                               unsigned char* slice, int tid, int tp, uint32_t rank) {
-  using A = Arith<Real>;
   using G = PairGeom<L>;
   constexpr int HL = G::HL, HP = G::HP, ZL = G::ZL, S = G::S;
   constexpr int NH = L * L * L / 2;  // sites per colour of the whole lattice
@@ -1783,7 +1769,6 @@ template <typename Real, int kL, int kRS>
 __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path,
                                   const SweepParams& P, unsigned char* slice, int tid, int tp,
                                   int bar, Real* lat_cta) {
-  using A = Arith<Real>;
   const int L = kL > 0 ? kL : sy.L, HL = L / 2, HP = L * L / 2;
   const int hps = StreamLayout<Real>::hps(L);
   const uint32_t bytes = static_cast<uint32_t>(hps * sizeof(Real));

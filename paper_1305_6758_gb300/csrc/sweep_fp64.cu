@@ -1,5 +1,6 @@
-// FP64 form of the shared-memory sweep (the plain FP64 GPU form): FP64 spins,
-// energy differences, Boltzmann factors and accumulators.
+// FP64 form of the shared-memory sweep: spins in 64-bit fixed point, moves decided
+// as FP64 energy differences and Boltzmann factors decide them (most already by
+// their FP32 values and error bound), FP64 accumulators.
 // This file holds part a (the smallest shared-memory lattice sizes) and the
 // host entry points; parts b, c and d are sweep_fp64_b.cu, _c.cu and _d.cu.
 #define REAL double
