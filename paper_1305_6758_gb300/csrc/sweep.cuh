@@ -497,7 +497,8 @@ static __device__ __noinline__ bool accept_exact(int64_t dx, int64_t dy, int64_t
 // lies outside the FP32 acceptance's error bound (all but about 1e-5 of the
 // moves; those take accept_exact), and the trial spin is evaluated to 2^-53 in
 // integers (fix_trial), by warps in which a move was accepted.  L = 16, three
-// temperatures of 1024 paths: 5.2e9 attempts/s with FP64 arithmetic, 7.3e10 so.
+// temperatures of 1024 paths: 5.2e9 attempts/s with FP64 arithmetic, 7.1e10 so in
+// thermalisation and 6.1e10 in measured sweeps.
 //
 // The FP32 stage of a move: the trial direction in units of 2^-28 and the uniform.
 struct FixDraw {
@@ -669,8 +670,7 @@ __device__ __forceinline__ void half_sweep(const Geom& geo, int c, const PhiloxP
       // Where chunks of two give a warp too few independent random-number
       // chains, the rounds of a thermalisation sweep are taken two at a time (u
       // and u + tp side by side; measurement sweeps keep the order of their FP32
-      // sums, and FP64 has no registers for it: 7.3e10 -> 4.7e10 attempts/s at
-      // L = 16).  Attempts/s before -> after, sweeps of all kinds: L = 10, 1000
+      // sums, and FP64 has no registers for it: a third slower at L = 16).  Attempts/s before -> after, sweeps of all kinds: L = 10, 1000
       // paths (7 warps per SM) 1.36e11 -> 1.47e11, a full GPU 2.08e11 ->
       // 2.15e11, L = 22 1.71e11 -> 1.72e11, L = 26 1.73e11 -> 1.85e11.  Chunks
       // of three lose by it (L = 6: 1.21e11 -> 1.18e11), four rounds at a time
@@ -1863,13 +1863,11 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
   group_sync(tp, bar);
 
   constexpr bool kFixedRows = kL > 0 && kRS > 0 && kL % kRS == 0;
-  // FP32 with three or four rows per thread (the planner's layouts): see phase
+  // FP32 with between three and four rows per thread (the planner's layouts): see phase
   constexpr bool kFourRows = sizeof(Real) == 4 && kRS == 0;
-  const bool four_rows = 3 * RS <= L && L <= 4 * RS;
+  const bool four_rows = stream_four_rows(L, RS);
   const int hp0 = hx + HL * y0;
-  StreamRow srow[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) srow[k] = stream_row(L, RS, y0, k);
+  const StreamRows srows = stream_rows(L, RS, y0);
   int accepted = 0;
   bool ok = true;
 
@@ -1970,14 +1968,14 @@ __device__ void run_path_streamed(const DevSystem& sy, int sys_idx, int64_t path
           auto rows = [&](auto meas_c, auto energy_c) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              const bool act = srow[k].act;
-              const int hp = hp0 + srow[k].off;
+              const StreamRow row = stream_row(srows, HL, RS, k);
+              const int hp = hp0 + row.off;
               const int xo = hp + (k & 1 ? xoc : xoa), p = k & 1 ? pc : pz;
-              const int yp = hp + srow[k].yp, ym = hp + srow[k].ym;
+              const int yp = hp + row.yp, ym = hp + row.ym;
               const V3<Real> f = add3(add3(add3(add3(add3(same.ld(hp), same.ld(xo)), same.ld(yp)), same.ld(ym)),
                                            up.ld(hp)), dn.ld(hp));
               update_spin<decltype(meas_c)::value, decltype(energy_c)::value>(
-                  static_cast<uint32_t>(2 * (hp + HP * z) + p), pre, P.key, own, hp, own.ld(hp), f, cp, act, accepted,
+                  static_cast<uint32_t>(2 * (hp + HP * z) + p), pre, P.key, own, hp, own.ld(hp), f, cp, row.act, accepted,
                   part);
             }
           };

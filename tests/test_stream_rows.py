@@ -1,9 +1,8 @@
 """The rows a thread of the streamed kernel walks, against the lattice (CPU).
 
 Every row lies in the half-plane and its +-y offsets lead to its periodic
-neighbours, also those of a row that stands in for one outside the lattice
-(three rows covering L exactly, L = 3 RS, among them): its spins are read, not
-used.  Each row of the lattice is acted on exactly once.
+neighbours, also those of a row that stands in for one outside the lattice: its
+spins are read, not used.  Each row of the lattice is acted on exactly once.
 """
 import os
 import shutil
@@ -35,6 +34,7 @@ def test_rows_stay_in_the_half_plane(tmp_path):
         assert y == (y0 + k * RS if act else y0), line
         if act:
             acted[L, RS].append(y)
-    assert any(L == 3 * RS for L, RS in acted) and any(L == 4 * RS for L, RS in acted)
+    assert any(L == 4 * RS for L, RS in acted) and any(3 * RS + 1 == L for L, RS in acted)
+    assert (30, 8) in acted and (28, 9) in acted and (60, 16) in acted  # default layouts
     for (L, _), rows in acted.items():
         assert sorted(rows) == list(range(L))
