@@ -27,10 +27,11 @@
 // (from the colour-1 counts, every bond once) and magnetisation are exact
 // integers; they enter the FP64 per-path accumulators of the Heisenberg
 // kernels' measurement ring, in the same record layout (m_x = m_y = 0, m_z = m).
-// What bounds it is instruction issue, Philox half of it.  L = 60, four T x
-// 10^4 paths: with a byte load per neighbour and 256 threads per path 38.6 ms for
-// 50 + 100 sweeps (5.6e11 attempts/s), 22.5 ms (9.6e11) with words and one warp
-// per path.
+// What bounds it is instruction issue, Philox half of it, and some spilled
+// registers (64 per thread, for CTAs of up to 1024; 100 bytes of spill stores, 192
+// of loads).  L = 60, four T x 10^4 paths: with a byte load per neighbour and 256
+// threads per path 38.6 ms for 50 + 100 sweeps (5.6e11 attempts/s), 21.8 ms (9.9e11)
+// with words and one warp per path.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -355,26 +356,35 @@ __global__ void __launch_bounds__(kIsingThreads, 1) ising_kernel(const SweepPara
 // whose strips fill its lanes best, weighed with the warps an SM then holds (of
 // 32; 13 reach 0.56, 26 0.94 of the rate, at L = 128) and with the barrier that
 // more than one warp per path needs (about 7%).  Attempts/s by threads per path:
-// L = 60 32: 1.02e12, 64: 9.3e11, 256: 6.5e11; L = 100 32: 7.9e11, 64: 9.3e11.
-int ising_threads(int L, int64_t paths_per_sm, int smem_max, int ring, int most) {
+// L = 60 32: 9.9e11, 64: 9.0e11, 256: 6.0e11; L = 100 32: 7.7e11, 64: 9.0e11, 128:
+// 9.2e11; L = 128 32: 6.4e11, 64: 9.8e11, 128: 1.02e12.
+// `full`: for a GPU full of paths; `loaded`: for paths_per_sm, at most `most`.  (In one
+// pass: the segment search takes some 10 us of a small call.)
+IsingThreads ising_threads(int L, int64_t paths_per_sm, int smem_max, int ring, int most) {
   const int S = (L / 2) * ((L + 3) / 4);
-  double best = -1.0;
-  int best_t = 32;
-  for (int t = 32; t <= most && (t == 32 || t < 2 * S); t += 32) {
+  double best_full = -1.0, best_loaded = -1.0;
+  IsingThreads best{32, 32};
+  for (int t = 32; t <= kIsingThreads && (t == 32 || t < 2 * S); t += 32) {
     const int slice = (slice_spin_offset(t, ring, kRedBytes) + ising_slice_spin_bytes(L) + 127) / 128 * 128;
-    int64_t fit = std::min<int64_t>(smem_max / slice, t > 32 ? std::min(15, kIsingThreads / t) : kIsingThreads / t);
-    fit = std::min(fit, paths_per_sm);
+    const int64_t fit = std::min<int64_t>(smem_max / slice, t > 32 ? std::min(15, kIsingThreads / t) : kIsingThreads / t);
     if (fit < 1) continue;
     const int q = ising_segment(L, t), units = (L / 2) * (((L + 3) / 4 + q - 1) / q);
     const double fill = S / (static_cast<double>(t) * ((units + t - 1) / t) * (q + 0.4));
-    const double rate = fill * std::pow(std::min(1.0, static_cast<double>(fit) * t / 1024.0), 0.65) *
-                        (t == 32 ? 1.0 : 0.93);
-    if (rate > best + 1e-9) {
-      best = rate;
-      best_t = t;
+    auto rate = [&](int64_t paths) {
+      return fill * std::pow(std::min(1.0, static_cast<double>(std::min(fit, paths)) * t / 1024.0), 0.65) *
+             (t == 32 ? 1.0 : 0.93);
+    };
+    const double full = rate(fit), loaded = rate(paths_per_sm);
+    if (full > best_full + 1e-9) {
+      best_full = full;
+      best.full = t;
+    }
+    if (t <= most && loaded > best_loaded + 1e-9) {
+      best_loaded = loaded;
+      best.loaded = t;
     }
   }
-  return best_t;
+  return best;
 }
 
 cudaError_t ising_prepare(int device, int* max_dynamic, int* max_threads) {

@@ -49,7 +49,10 @@ constexpr int kStreamL64 = -1064;
 
 // The square-lattice Ising kernel (any even L, sizes mixed or not).
 constexpr int kIsingKernel = -3;
-int ising_threads(int L, int64_t paths_per_sm, int smem_max, int ring, int most);
+struct IsingThreads {
+  int full, loaded;
+};
+IsingThreads ising_threads(int L, int64_t paths_per_sm, int smem_max, int ring, int most);
 cudaError_t ising_prepare(int device, int* max_dynamic, int* max_threads);
 cudaError_t ising_occupancy(int cta, int smem, int* blocks);
 cudaError_t launch_ising(const SweepParams& p, int grid, int cta, int smem, cudaStream_t st);

@@ -608,23 +608,27 @@ int plan(mp_state* h, const mp_config* cfg) {
     // depend on the number of threads, which is chosen by the paths that an SM
     // gets; it does depend on the ring (the sweeps summed together), which is
     // therefore that of the threads chosen for a full GPU.
-    std::function<int(int64_t, int, int)> by_load;  // threads for so many paths per SM, this ring, at most so many
+    const int64_t load = (batch_paths + sms - 1) / sms;  // paths per SM
+    std::function<int(bool, int)> by_load;  // threads for a full GPU (true) or for `load`, with this ring
+    IsingThreads ising{};                   // both, with a ring of 16
     if (h->systems[k].lattice == MP_LATTICE_ISING) {
-      by_load = [&](int64_t per_sm, int r, int most) {
-        return ising_threads(h->systems[k].L, per_sm, smem_max, r, most);
+      by_load = [&](bool full, int r) {
+        if (full) ising = ising_threads(h->systems[k].L, load, smem_max, 16, tp_max);
+        if (full) return ising.full;
+        return r == 16 ? ising.loaded : ising_threads(h->systems[k].L, load, smem_max, r, tp_max).loaded;
       };
     } else if (h->systems[k].lattice == MP_LATTICE_SC && real == 8) {
       // FP64 lattices are large (L = 16: two paths per SM): the count that fills
-      // its own lanes best, weighed with the warps the SM then holds (of 16).  L =
-      // 16, 3072 paths: 6.2e10 attempts/s with 128 threads, 7.3e10 with 256; L = 20,
-      // 500 paths: 3.4e10 with 160, 6.2e10 with 512.
-      by_load = [&](int64_t per_sm, int r, int most) {
+      // its own lanes best, weighed with the warps the SM then holds (of 16).  Half
+      // the sweeps measured, L = 16, 3072 paths: 5.7e10 attempts/s with 128 threads,
+      // 6.5e10 with 256; L = 20, 500 paths: 3.1e10 with 160, 5.4e10 with 512.
+      by_load = [&](bool full, int r) {
         double best = -1.0;
         int best_t = 0;
-        for (int c = 32; c <= std::min(most, round_up(NH, 32)); c += 32) {
+        for (int c = 32; c <= std::min(full ? cta_max : tp_max, round_up(NH, 32)); c += 32) {
           const int units = h->systems[k].L * h->systems[k].L / 2 * column_segments(h->systems[k].L, 1, c);
           int64_t fit = std::min<int64_t>(smem_max / need_of(c, r), c > 32 ? std::min(15, cta_max / c) : cta_max / c);
-          fit = std::min(fit, per_sm);
+          if (!full) fit = std::min(fit, load);
           if (fit < 1) continue;
           const double rate = units / (static_cast<double>((units + c - 1) / c) * c) *
                               std::min(1.0, static_cast<double>(fit) * c / 512.0);
@@ -636,7 +640,7 @@ int plan(mp_state* h, const mp_config* cfg) {
         return best_t;
       };
     }
-    if (t == 0 && by_load) t = by_load(INT64_MAX, h->systems[k].lattice == MP_LATTICE_ISING ? 16 : 1, cta_max);
+    if (t == 0 && by_load) t = by_load(true, 1);
     if (t == 0 && h->systems[k].lattice == MP_LATTICE_SC) {
       // a divisor of the sites per colour lets each thread walk a block of
       // columns; pick the one closest to the target sites per thread
@@ -657,7 +661,7 @@ int plan(mp_state* h, const mp_config* cfg) {
     ring[k] = 16;
     pick_ring(ring[k], slice[k], [&]() { return need_of(t, ring[k]); }, t);
     if (by_default && by_load) {
-      const int loaded = by_load((batch_paths + sms - 1) / sms, ring[k], tp_max);
+      const int loaded = by_load(false, ring[k]);
       if (loaded > 0) {
         t = loaded;
         slice[k] = need_of(t, ring[k]);
