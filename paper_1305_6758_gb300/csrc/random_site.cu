@@ -394,8 +394,8 @@ __global__ void __launch_bounds__(32 * kWarps) random_site_kernel(const SweepPar
 
 // One thread per path, for many paths of very few sites (N <= kThreadSites),
 // where 32 attempts of one path hardly ever act together: chain of 8, 10^4
-// paths, FP32: 3.3e10 attempts/s against 2.2e10 by warps, measured sweeps
-// 1.4e10 against 0.5e10; with 10^6 paths 1.6e11 against 2.7e10.  Lattices in HBM,
+// paths, FP32: 4.5e10 attempts/s against 2.3e10 by warps, measured sweeps
+// 2.1e10 against 0.5e10; with 10^6 paths 1.8e11 against 2.5e10.  Lattices in HBM,
 // element (site i, path p) of system k at spin_offset[k] / 3 + i * P_k + p, so
 // that a warp's threads read consecutive elements of the same site.
 constexpr int kThreadSites = 16;  // and enough paths for a warp of them on every SM

@@ -1184,7 +1184,7 @@ __device__ __forceinline__ int* cancel_flags() {
 // attempts, most of it in their random numbers and trial spins, which do not
 // depend on the lattice: both colours' are drawn together, before the first
 // update, and neighbours are decoded once per path.
-// FP64 L = 4, 256 paths: 1.31 -> 0.93 us per sweep; FP32 with 2000 paths 9.9e10 -> 1.3e11
+// FP64 L = 4, 256 paths: 1.31 -> 0.98 us per sweep; FP32 with 2000 paths 9.9e10 -> 1.3e11
 // attempts/s.
 //
 // FP32 sums depend on their order, which is that of tm threads each taking its
