@@ -670,8 +670,9 @@ __device__ __forceinline__ void half_sweep(const Geom& geo, int c, const PhiloxP
       // Where chunks of two give a warp too few independent random-number
       // chains, the rounds of a thermalisation sweep are taken two at a time (u
       // and u + tp side by side; measurement sweeps keep the order of their FP32
-      // sums, and FP64 has no registers for it: a third slower at L = 16).  Attempts/s before -> after, sweeps of all kinds: L = 10, 1000
-      // paths (7 warps per SM) 1.36e11 -> 1.47e11, a full GPU 2.08e11 ->
+      // sums, and FP64 has no registers for it: a third slower at L = 16).
+      // Attempts/s before -> after, sweeps of all kinds: L = 10, 1000 paths (7
+      // warps per SM) 1.36e11 -> 1.47e11, a full GPU 2.08e11 ->
       // 2.15e11, L = 22 1.71e11 -> 1.72e11, L = 26 1.73e11 -> 1.85e11.  Chunks
       // of three lose by it (L = 6: 1.21e11 -> 1.18e11), four rounds at a time
       // lose everywhere.
@@ -1203,7 +1204,8 @@ __device__ __forceinline__ void run_path(const Geom geo, const DevSystem& sy, in
                                          int tid, int tp, int bar, Real* hbm_spins = nullptr) {
   static_assert(!kWide || (sizeof(Real) == 4 && Geom::kColumns && !kOne), "wide paths are FP32 column walks");
   constexpr bool kExact = kExactSums<Real, Geom>;
-  Real* sp = hbm_spins ? hbm_spins : reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring, kExact ? kRedBytesFix : kRedBytes));
+  Real* sp = hbm_spins;
+  if (!sp) sp = reinterpret_cast<Real*>(slice + slice_spin_offset(tp, sy.ring, kExact ? kRedBytesFix : kRedBytes));
   const int S = geo.stride();
   const uint32_t c2 = static_cast<uint32_t>(sy.path_begin + path);  // path id
   const uint32_t c3u = kTagUpdate | (static_cast<uint32_t>(sys_idx) << 8);
