@@ -386,9 +386,10 @@ int mp_system_plan(mp_handle h, int system, int* threads_per_path, int* paths_pe
  * ranges of the same systems and seed): gather their records in path order
  * and reduce them here to obtain exactly the estimates of one process
  * running every path (all with the same threads_per_path, 0 included, and
- * without MP_FLAG_AUTOTUNE, whose choice depends on n_paths).  Allocates and frees a small device table (and, for
- * systems of more than MP_R_MAX_PATHS paths, 2 x paths doubles of sort
- * space) and synchronises `stream` (cudaStream_t; NULL = legacy default).
+ * without MP_FLAG_AUTOTUNE, whose choice depends on n_paths).  Allocates and
+ * frees a small device table, paths + 64 n_systems doubles of scratch (and, for
+ * systems of more than MP_R_MAX_PATHS paths, 2 x paths doubles of sort space)
+ * and synchronises `stream` (cudaStream_t; NULL = legacy default).
  * Errors: MP_EINVAL (NULL pointer, bad system), MP_ENOMEM, MP_ECUDA; the text
  * is mp_last_error(NULL). */
 int mp_reduce(const mp_system* systems, int n_systems, int64_t n_therm, int64_t n_meas,

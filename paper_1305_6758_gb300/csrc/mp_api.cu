@@ -1387,6 +1387,8 @@ int mp_estimates(mp_handle h, int system, mp_estimates_t* out) {
       return error_status(h, flag);
     }
     h->est_run = h->runs;
+  } else {
+    MP_CUDA(h, cudaStreamSynchronize(h->stream));  // as every call that returns host data
   }
   std::memcpy(out, &h->est_host[static_cast<size_t>(system) * MP_NEST], sizeof(mp_estimates_t));
   out->elapsed_s = h->est_elapsed;
