@@ -120,14 +120,14 @@ BYTES_PER_ATTEMPT_FP32 = 24
 # with this hash (sha256 over csrc/, first 16 hex digits); any change of the
 # sources voids it and the roofline reports traffic null.  Each is the timed
 # launch of the workload's bench command, captured at full size (one ncu pass):
-# sc16 reads 1.1 MB (tables; the lattices stay in shared memory), batched
-# 0.65 MB (every size, L = 32 included, stays in shared memory), large moves
-# 28.95 TB against 28.99 TB of algorithmic bytes, ising 0.48 MB.
+# sc16 reads 1.3 MB (tables; the lattices stay in shared memory), batched
+# 0.64 MB (every size, L = 32 included, stays in shared memory), large moves
+# 28.94 TB against 28.99 TB of algorithmic bytes, ising 0.46 MB.
 TRAFFIC = {
-    "sc16": {"sources": "6b0a8cd5a7585476", "bytes": 1.146624e6},
-    "large": {"sources": "6b0a8cd5a7585476", "bytes": 14.445352921344e12 + 14.501790765824e12},
-    "batched": {"sources": "6b0a8cd5a7585476", "bytes": 0.652544e6},
-    "ising": {"sources": "6b0a8cd5a7585476", "bytes": 0.396800e6 + 0.086272e6},
+    "sc16": {"sources": "1575d747cd87de05", "bytes": 1.269504e6},
+    "large": {"sources": "1575d747cd87de05", "bytes": 14.436410070272e12 + 14.503800877824e12},
+    "batched": {"sources": "1575d747cd87de05", "bytes": 0.639232e6},
+    "ising": {"sources": "1575d747cd87de05", "bytes": 0.370944e6 + 0.084992e6},
 }
 
 
